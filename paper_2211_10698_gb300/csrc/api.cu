@@ -72,6 +72,8 @@ struct ccm_case_s {
   double* dpart;
   unsigned int* bar_count;
   unsigned long long* fxacc;  // words of the fixed-point reduce-barrier (pcg_fixed.cuh)
+  ulonglong2* mail;           // mailboxes of the resident tiles (pcg_fused.cu), mail_slots of them
+  size_t mail_slots = 0;
   int* bar_err;
   DevStats* ds;
   bool geometry = false;
@@ -182,6 +184,8 @@ void carve(ccm_case c, Carver& cv) {
   c->fout = cv.take<double>(4);
   c->bar_count = cv.take<unsigned int>(kBarWords);
   c->fxacc = cv.take<unsigned long long>(kFxAccWords);
+  c->mail_slots = fused_mail_slots_max(c->g.nx, c->g.ny);
+  c->mail = cv.take<ulonglong2>(c->mail_slots);
   c->bar_err = cv.take<int>(4);
   c->ds = cv.take<DevStats>(1);
   c->hs_u = cv.take<double>(N);
@@ -302,6 +306,8 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
     FusedSolve f{};
     f.a = scaled_solve_of(v, x, b, c->pz, nullptr, nullptr, c->pp0, nullptr);
     f.fxacc = c->fxacc;
+    f.mail = c->mail;
+    f.mail_slots = c->mail_slots;
     f.fx_fallback_every = c->fx_fallback_every;
     f.a.partials = c->partials;
     f.a.bar = case_barrier(c);
@@ -530,6 +536,8 @@ ccm_status autotune_poisson(ccm_case c) {
     FusedSolve f{};
     f.a = scaled_solve_of(v, x, b, c->pz, nullptr, nullptr, c->pp0, nullptr);
     f.fxacc = c->fxacc;
+    f.mail = c->mail;
+    f.mail_slots = c->mail_slots;
     f.a.partials = c->partials;
     f.a.bar = case_barrier(c);
     f.a.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, nullptr, nullptr};

@@ -97,31 +97,39 @@ cudaError_t run_poisson_scaled(const ScaledSolve& a, cudaStream_t st);
 // The same solve with one grid barrier per iteration (pcg_fused.cu): 2-D tiles, the ring of
 // each tile recomputed by its block, r, w, s double-buffered.  a.xs and a.p are used, a.r,
 // a.w, a.s are not.
-// Words of the fixed-point reduce-barrier (pcg_fixed.cuh): three rotating buffers of kFxWords
+// Words of the fixed-point reduce-barrier (pcg_fixed.cuh): two alternating buffers of kFxWords
 // 64-bit words, each word on its own 128-byte line.
 constexpr int kFxWords = 16;
 constexpr int kFxStride = 16;
-constexpr int kFxAccWords = 3 * kFxWords * kFxStride;
+constexpr int kFxAccWords = 2 * kFxWords * kFxStride;
 
 struct FusedSolve {
   ScaledSolve a;
   unsigned long long* fxacc;  // kFxAccWords words (cleared by the kernel itself)
   int fx_fallback_every;      // tests only: every k-th reduction takes the FP64 fallback (0: on overflow only)
-  double* R[2];
+  double* R[2];               // resident tiles use R[0] only
   double* W[2];
   double* S[2];
+  ulonglong2* mail;         // resident tiles: mailboxes, mail_slots 16-byte slots (cleared by the kernel itself)
+  size_t mail_slots;
   int TX, TY, nbx, ntiles;  // tile plan; TX = 0 lets the launcher choose
-  int list_cap;             // set by the launcher: entries of the per-tile list of non-uniform cells
   int resident;             // 1: each tile keeps its vectors in shared memory (k_pcg_poisson_f2)
-  int lcache;               // set by the launcher (resident): the listed cells' coefficients cached in shared memory
+  // set by the launcher
+  int wx;                   // TX clipped to the grid's width
+  int list_cap;             // entries of the per-tile list of non-uniform cells
+  int lcache;               // (resident) the first listed cells' coefficients cached in shared memory
+  int dcache;               // (resident) room for every cell's coefficients in shared memory
+  int defer;                // (resident) a second r frame, so that p waits for the barrier as x does
 };
+constexpr int kFusedTilesMax = 512;  // tiles of a launch, at most (two per SM)
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
 void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles);
 int fused_blocks();
-size_t fused_resident_smem(int TX, int TY, bool cache);
-bool fused_resident_fits(int TX, int TY, int ntiles, bool cache);
-int fused_resident_fit(int TX, int TY, int ntiles);
+size_t fused_resident_smem_min(int TX, int TY);
 bool fused_resident_ok(int TX, int TY, int ntiles);
+// Mailbox slots of a resident plan, and of any resident plan of a grid.
+size_t fused_mail_slots(int nx, int TX, int TY, int ntiles);
+size_t fused_mail_slots_max(int nx, int ny);
 
 // The same solve for small grids inside one thread-block cluster (pcg_cluster.cu).
 struct ClusterSolve {

@@ -28,10 +28,17 @@
 // more than 2^kFxMargin-fold in one iteration, or is not finite) is counted in an extra
 // word; every block then sees the count and repeats the reduction in FP64 (the fallback).
 //
-// Three buffers of words rotate by reduction index: block 0 clears the buffer of reduction
-// i - 1 after the wait of reduction i (every block read it before adding to reduction i), and
-// that clearing precedes block 0's release for reduction i + 1, which every block acquires
-// before it adds to reduction i + 2, the next user of the buffer.
+// Two buffers of words alternate by reduction index and are never cleared during a solve: a
+// block keeps each buffer's last complete words and takes the difference, in which counts and
+// digit sums both come out modulo 2^64.  A block adds to reduction i + 2 only after its wait of
+// reduction i + 1, to which every block has added only after its own wait of reduction i, so no
+// word of reduction i changes while a block still reads it.
+//
+// The words carry all that the reduction needs.  Where other data must be visible after the
+// wait (vectors in global memory that other blocks read), the arrival is a release and the
+// wait an acquire; where neighbours exchange their data in tagged slots (tag_put, tag_get
+// below) both are relaxed, which takes the wait for the block's outstanding stores out of
+// every iteration.
 #pragma once
 #include <cstring>
 
@@ -101,19 +108,30 @@ __host__ __device__ __forceinline__ bool fx_digits(double v, int lo, int (&d)[kF
     m |= 1ULL << 52;
     e = ex - 1075;
   }
-  const int s = e - lo;  // position of m's lowest bit in the window
+  int s = e - lo;  // position of m's lowest bit in the window
   const bool ok = ex != 0x7ff && (m == 0 || s + 53 <= kFxTop);
-  unsigned __int128 X = 0;
-  if (ok && m != 0) {
-    if (s >= 0) X = (unsigned __int128)m << s;
-    else if (s > -64) X = (unsigned __int128)(m >> (-s));
+  if (!ok) m = 0;
+  if (s < 0) {
+    m = s > -64 ? m >> -s : 0;
+    s = 0;
   }
-  const bool neg = (b >> 63) != 0;
-#pragma unroll
-  for (int k = 0; k < kFxDigits; ++k) {
-    const int dk = (int)((unsigned long long)(X >> (kFxBits * k)) & ((1ULL << kFxBits) - 1));
-    d[k] = neg ? -dk : dk;
+  // m (53 bits) shifted by the offset in its lowest digit covers three digits, w0 .. w0 + 2
+  static_assert(kFxBits == 26 && kFxDigits == 5 && kFxTop <= 108, "three digits, the lowest of them one of 0, 1, 2");
+  const int w0 = s >= 2 * kFxBits ? 2 : (s >= kFxBits ? 1 : 0), off = s - kFxBits * w0;
+  constexpr unsigned int mask = (1u << kFxBits) - 1;
+  int p0 = (int)((unsigned int)(m << off) & mask);
+  int p1 = (int)((unsigned int)(m >> (kFxBits - off)) & mask);
+  int p2 = (int)(unsigned int)((m >> (kFxBits - off)) >> kFxBits);
+  if (b >> 63) {
+    p0 = -p0;
+    p1 = -p1;
+    p2 = -p2;
   }
+  d[0] = w0 == 0 ? p0 : 0;
+  d[1] = w0 == 0 ? p1 : (w0 == 1 ? p0 : 0);
+  d[2] = w0 == 0 ? p2 : (w0 == 1 ? p1 : p0);
+  d[3] = w0 == 1 ? p2 : (w0 == 2 ? p1 : 0);
+  d[4] = w0 == 2 ? p2 : 0;
   return ok;
 }
 
@@ -159,24 +177,52 @@ __host__ __device__ __forceinline__ double fx_value(const long long* S, int lo) 
   return neg ? -r : r;
 }
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+// Loads of a polled word: acquire, or relaxed where the word itself is all that is read.
+template <bool ACQ>
+__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
   unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  if constexpr (ACQ) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 
-// Shared state of one block's fixed-point reduction.
+// A value and its tag in one 16-byte slot, written and read as one 128-bit access: a reader
+// that finds the tag it expects has the value that was stored with it, whatever else is in
+// flight, so neighbours exchange values without a fence.
+__device__ __forceinline__ void tag_put(ulonglong2* slot, double v, unsigned int tag) {
+  const unsigned __int128 w = ((unsigned __int128)tag << 64) | (unsigned long long)__double_as_longlong(v);
+  asm volatile("st.relaxed.gpu.global.b128 [%0], %1;" ::"l"(slot), "q"(w) : "memory");
+}
+// true with the slot's value in v if it carries `tag`
+__device__ __forceinline__ bool tag_get(const ulonglong2* slot, unsigned int tag, double& v) {
+  unsigned __int128 w;
+  asm volatile("ld.relaxed.gpu.global.b128 %0, [%1];" : "=q"(w) : "l"(slot) : "memory");
+  v = __longlong_as_double((long long)(unsigned long long)w);
+  return (unsigned long long)(w >> 64) == tag;
+}
+
+// tag_get until the slot carries `tag`, within `budget` cycles (else *err is raised and false returned)
+__device__ __forceinline__ bool tag_wait(const ulonglong2* slot, unsigned int tag, double& v, long long budget,
+                                         int* err) {
+  const long long t0 = clock64();
+  while (!tag_get(slot, tag, v)) {
+    if (clock64() - t0 > budget) {
+      atomicExch(err, 1);
+      return false;
+    }
+  }
+  return true;
+}
+
+// Shared state of one block's fixed-point reduction: per-warp digit sums of NT threads.
+template <int NT>
 struct FxShared {
-  int w[kPcgThreads / 32][kFxWords];  // per-warp digit sums
-  long long s[kFxWords];              // the grid's digit sums (and the overflow count)
-  int ok;                             // 0: the wait ran out
+  int w[NT / 32][kFxWords];
 };
 
-// Arrival: the block's digits of v[0..2] for reduction buffer `buf` (all threads).  Every
-// thread's writes before the call are released with the block's words.
+// The digits of v[0..2] summed per warp into sh (each of the NT threads).
 template <int NT>
-__device__ __forceinline__ void fx_arrive(const double (&v)[4], int lo, unsigned long long* acc, int buf, int absent,
-                                          FxShared& sh) {
+__device__ __forceinline__ void fx_block_digits(const double (&v)[4], int lo, FxShared<NT>& sh) {
   int d[kFxWords];
   bool fit = true;
 #pragma unroll
@@ -193,51 +239,50 @@ __device__ __forceinline__ void fx_arrive(const double (&v)[4], int lo, unsigned
   if (lane == 0)
 #pragma unroll
     for (int k = 0; k < kFxWords; ++k) sh.w[wid][k] = d[k];
-  __syncthreads();
-  if (threadIdx.x < kFxWords) {
+}
+
+// Arrival, by one whole warp after every warp's digits are in sh: the block's digit sums added
+// to the words of buffer `buf`.  REL: what the warp has seen (its barrier with the others
+// included) is released with the words.
+template <int NT, bool REL>
+__device__ __forceinline__ void fx_arrive(unsigned long long* acc, int buf, bool absent, const FxShared<NT>& sh) {
+  const int lane = threadIdx.x & 31;
+  if (lane < kFxWords) {
     long long s = 0;
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) s += sh.w[w][threadIdx.x];
+    for (int w = 0; w < NT / 32; ++w) s += sh.w[w][lane];
     const unsigned long long word = (1ULL << kFxCountShift) + (unsigned long long)(s + kFxBias);
-    unsigned long long* dst = acc + ((size_t)buf * kFxWords + threadIdx.x) * kFxStride;
-    if ((int)blockIdx.x != absent) asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(word) : "memory");
+    unsigned long long* dst = acc + ((size_t)buf * kFxWords + lane) * kFxStride;
+    if (!absent) {
+      if constexpr (REL) asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(word) : "memory");
+      else asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(word) : "memory");
+    }
   }
 }
 
-// Wait: until every block has added to every word of buffer `buf` (bounded by `budget`
-// cycles; on give-up *err is raised and false returned), then the grid's digit sums in
-// sh.s.  Block 0 then clears buffer `clear`.  All threads.
-__device__ __forceinline__ bool fx_wait(unsigned long long* acc, int buf, int clear, long long budget, int* err,
-                                        FxShared& sh) {
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const unsigned long long* src = acc + ((size_t)buf * kFxWords + (lane < kFxWords ? lane : 0)) * kFxStride;
-    const unsigned long long nb = gridDim.x;
-    unsigned long long w = 0;
-    bool done = lane >= kFxWords;
-    int ok = 1;
-    const long long t0 = clock64();
-    while (true) {
-      if (!done) {
-        w = ld_acquire_u64(src);
-        done = (w >> kFxCountShift) == nb;
-      }
-      if (__all_sync(0xffffffffu, done)) break;
-      if (__shfl_sync(0xffffffffu, clock64() - t0 > budget ? 1 : 0, 0)) {
-        ok = 0;
-        break;
-      }
+// Wait, by one whole warp: until all nb blocks have added to every word of buffer `buf`
+// (bounded by `budget` cycles; on give-up *err is raised and false returned).  last: this lane's
+// word of that buffer after its previous use (0 at first), updated.  digit: the grid's sum of
+// this lane's word (lanes below kFxWords).
+template <bool ACQ>
+__device__ __forceinline__ bool fx_wait(const unsigned long long* acc, int buf, int nb, long long budget, int* err,
+                                        unsigned long long& last, long long& digit) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long* src = acc + ((size_t)buf * kFxWords + (lane < kFxWords ? lane : 0)) * kFxStride;
+  unsigned long long w = 0, d = 0;
+  const long long t0 = clock64();
+  while (true) {
+    w = ld_word<ACQ>(src);
+    d = w - last;
+    if (__all_sync(0xffffffffu, (d >> kFxCountShift) == (unsigned long long)nb)) break;
+    if (__shfl_sync(0xffffffffu, clock64() - t0 > budget ? 1 : 0, 0)) {
+      if (lane == 0) atomicExch(err, 1);
+      return false;
     }
-    if (lane < kFxWords)
-      sh.s[lane] = (long long)(w & ((1ULL << kFxCountShift) - 1)) - (long long)nb * kFxBias;
-    if (lane == 0) {
-      sh.ok = ok;
-      if (!ok) atomicExch(err, 1);
-    }
-    if (ok && blockIdx.x == 0 && lane < kFxWords) acc[((size_t)clear * kFxWords + lane) * kFxStride] = 0ULL;
   }
-  __syncthreads();
-  return sh.ok != 0;
+  last = w;
+  digit = (long long)(d & ((1ULL << kFxCountShift) - 1)) - (long long)nb * kFxBias;
+  return true;
 }
 
 }  // namespace ccm

@@ -24,86 +24,144 @@
 // shape that makes the largest tile smallest.
 //
 // Two instantiations of the same iteration: k_pcg_poisson_f1 keeps x~, r, p, s and w in global
-// memory (L2); k_pcg_poisson_f2 keeps its tile's x~, r, p, s, w and row kinds in shared memory
-// for the whole solve.  Only the tile's perimeter cells are read by other blocks (for their
-// ring), so f2 publishes r, w and s of its perimeter to the double-buffered global arrays once
-// per iteration and touches nothing else in global memory until the final x~ -> x.  Its
-// x~ += alpha p_i, which no other block reads, runs between the block's arrival at the grid
-// barrier and its wait, in the time the barrier would otherwise idle.
+// memory (L2) and publishes r, w and s there; k_pcg_poisson_f2 keeps its tile's x~, r, p, s, w
+// and row kinds in shared memory for the whole solve.  f2's ring needs one value per cell and
+// iteration from the neighbours: w.  The ring's r and s are kept by the tile that reads them,
+// updated with the same recurrences as their owner's (equal bit for bit), so a tile pushes the w
+// of its perimeter into its neighbours' mailboxes (one 16-byte slot per ring cell holding the
+// value and the iteration's number, double-buffered by parity) and reads its own mailbox.  The
+// slot's tag says that the value is there, and the words of the reduction carry the sums, so no
+// release or acquire, and no wait for outstanding stores, is left in f2's iteration.
+//
+// One further warp per block (the communication warp) sums the block's digits, adds them to the
+// reduction's words, waits for the grid's and forms the scalars of the next iteration in integer
+// arithmetic (pcg_scalar.cuh), while the other warps do the work that no other block reads:
+// p = r_i + beta p and x~ += alpha p (f2; r_i is kept beside r_{i+1} in a second framed copy,
+// where the tile leaves room for it: otherwise p is formed in step 1 and only x~ waits), and the
+// wait for the ring's next w.  The FP64 pipe (one warp instruction per 64 cycles on each
+// sub-partition) stays with the vectors, and the serial chain beside it.
+//
 // The sums of the iterations (reductions 1, 2, ...) are exact fixed-point sums that travel
 // with the grid barrier (pcg_fixed.cuh): the block's arrival adds its digit sums to words in
 // global memory and the wait on those words ends with the grid's sums in hand, so neither the
 // block sum nor the grid sum is a chain of FP64 additions.  Reduction 0 (phase 0) and the
 // rare reduction whose values leave the fixed-point window take the FP64 sums.
+//
+// What bounds it: on 1024x512 the FP64 pipe (10 operations per cell: 8.4 us of the 10.9 us per
+// iteration; 12.7 us with published r, w and s, release and acquire, and FP64 scalars), on small
+// grids the chain of one iteration: step, stencil, digits, one L2 hop between SMs (907 cycles
+// measured), scalars (128x64: 3.3 us per iteration against 4.3 us).
+//
+// Threads: NT = 128, 256 or 512 by the tile's cells (fused_threads), one to ten rows of the tile
+// each, so that a small tile is not paced by the block sums and barriers of idle warps.
 #include <algorithm>
 
 #include "pcg_common.cuh"
-#include "pcg_fixed.cuh"
+#include "pcg_scalar.cuh"
 
 namespace ccm {
 
 namespace {
 
-constexpr int kNT = 512;  // threads per block
+// Shared memory of a block besides the tile (dynamic).
+template <int NT>
+struct FusedShared {
+  double red[4][NT];
+  double bsum[8];
+  double gsum[8];
+  double alpha, beta, rr, bb;
+  int stop, lo, redo, fail;
+  int scan[NT / 32 + 1];
+  FxShared<NT> fx;
+};
 
+// Named barrier 2 hands the block's digits to the communication warp (which alone waits).
+template <int NT>
+__device__ __forceinline__ void digits_ready(bool wait) {
+  if (wait) asm volatile("bar.sync 2, %0;" ::"n"(NT + 32) : "memory");
+  else asm volatile("bar.arrive 2, %0;" ::"n"(NT + 32) : "memory");
+}
+
+// One tile of a solve: tile `tile` of the case's f.ntiles, one block of NT + 32 threads each.
 // RES: the tile's vectors live in shared memory (f2); otherwise in global memory (f1).
-template <bool RES>
-__device__ __forceinline__ void fused_body(const FusedSolve& f) {
-  __shared__ double red[4][kNT];
-  __shared__ double bsum[8];
-  __shared__ double gsum[8];
-  __shared__ double sc_alpha, sc_beta, sc_igamma, sc_den, sc_rr, sc_bb;
-  __shared__ double sc_igamma_next, sc_den_next;
-  __shared__ int sc_it, sc_stop;
-  __shared__ FxShared fxs;
-  // dynamic shared memory: with RES x~, p, s, w of the tile (TX*TY each) and r~ of the tile in
-  // a one-cell frame ((TX+2)*(TY+2), the frame holding the ring), then the ring
-  // [W: TY][E: TY][S: TX][N: TX] (used without RES), then with RES the tile's row kinds, then
-  // the list, then with RES and f.lcache the five scaled coefficients of the first kNT listed
-  // cells (8-byte aligned: TX is a multiple of 32)
+template <bool RES, int NT>
+__device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, FusedShared<NT>& sh) {
+  // dynamic shared memory: with RES x~, p, s, w of the tile (TX*TY each), r~ of the tile in a
+  // one-cell frame ((TX+2)*(TY+2), the frame holding the ring), with f.defer twice, then the
+  // ring's s [W: TY][E: TY][S: TX][N: TX] (without RES: the ring's r), then with RES and f.dcache
+  // the five scaled coefficients of every cell, with RES and f.lcache those of the first NT listed
+  // cells, then the list
   extern __shared__ double dyn[];
   unsigned int target = 0;
   const ScaledSolve& a = f.a;
-  const int nb = gridDim.x;
-  const Geom g = a.g;
+  const int nb = f.ntiles;
+  const Geom& g = a.g;
   const int nx = g.nx, ny = g.ny, P = g.pitch;
   const int TX = f.TX, TY = f.TY;
-  const bool active = (int)blockIdx.x < f.ntiles;
-  const int bx = blockIdx.x % f.nbx, by = blockIdx.x / f.nbx;
+  const int bx = tile % f.nbx, by = tile / f.nbx;
   const int i0 = bx * TX, j0 = by * TY;
-  const int i1 = active ? min(i0 + TX, nx) : i0, j1 = active ? min(j0 + TY, ny) : j0;
-  const int tx = threadIdx.x % TX, ty0 = threadIdx.x / TX, RP = kNT / TX;
+  const int i1 = min(i0 + TX, nx), j1 = min(j0 + TY, ny);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const bool comm = t >= NT;  // the communication warp
+  const int tx = t % TX, ty0 = t / TX, RP = NT / TX;
   const int ci = i0 + tx;  // this thread's column
-  const bool col = ci < i1;
   const int TXY = TX * TY;
+  // this thread's own cells: column ci, rows j0 + ty0 + q RP, q < nq; tile-local index t + q NT
+  const int nq = !comm && ci < i1 && j0 + ty0 < j1 ? (j1 - j0 - ty0 + RP - 1) / RP : 0;
+  const size_t k0 = g.idx(ci, j0 + ty0);  // of own cell 0 (used where nq > 0)
+  const size_t kstep = (size_t)RP * P;
   double* const sx = dyn;  // the RES arrays (unused otherwise)
   double* const sp = dyn + TXY;
   double* const ss = dyn + 2 * TXY;
   double* const sw = dyn + 3 * TXY;
   // RES: r~ of the tile with a one-cell frame that holds the ring, so that the stencil reads
-  // every neighbour from one array without a branch
-  const int TXP = TX + 2;
-  double* const sr = dyn + 4 * TXY;
-  double* const ring = RES ? dyn + 4 * TXY + TXP * (TY + 2) : dyn;
-  int8_t* const skind = reinterpret_cast<int8_t*>(ring + 2 * (TX + TY));
-  // tile-local index of own cell (i, j)
-  auto lidx = [&](int i, int j) -> int { return (j - j0) * TX + (i - i0); };
+  // every neighbour from one array without a branch; with defer two of them alternate
+  const int TXP = TX + 2, FR = TXP * (TY + 2);
+  const int lp0 = (ty0 + 1) * TXP + tx + 1, lpstep = RP * TXP;  // frame index of own cell 0, and step
+  const bool defer = RES && f.defer != 0;
+  double* sr = dyn + 4 * TXY;                         // r_i
+  double* srn = defer ? sr + FR : sr;                 // r_{i+1}
+  double* const ring = RES ? dyn + 4 * TXY + (defer ? 2 : 1) * FR : dyn;
+  double* const dcoef = ring + 2 * (TX + TY);
+  double* const lcoef = dcoef + (RES && f.dcache ? 5 * TXY : 0);
+  int* const list = reinterpret_cast<int*>(lcoef + (RES && f.lcache ? 5 * NT : 0));
   // index of cell (i, j) of the tile or its frame in the framed r~ (RES)
   auto lpad = [&](int i, int j) -> int { return (j - j0 + 1) * TXP + (i - i0 + 1); };
-  // own cells on the tile's perimeter are read by the neighbouring tiles' rings
-  auto perimeter = [&](int i, int j) -> bool { return i == i0 || i == i1 - 1 || j == j0 || j == j1 - 1; };
-  // ring cells: W and E columns, then S and N rows, taken by threads t, t + kNT, ...
+  // ring cells: W and E columns, then S and N rows, taken by threads t, t + NT, ...
   const int nring = 2 * (j1 - j0) + 2 * (i1 - i0);
-  // cell (ri, rj) of ring position t and its slot in `ring`; false outside the domain,
+  // cell (ri, rj) of ring position q and its slot in `ring`; false outside the domain,
   // where the value is 0
-  auto ring_cell = [&](int t, int& ri, int& rj, int& slot) -> bool {
+  auto ring_cell = [&](int q, int& ri, int& rj, int& slot) -> bool {
     const int h = j1 - j0, w = i1 - i0;
-    if (t < h) { ri = i0 - 1; rj = j0 + t; slot = t; }
-    else if ((t -= h) < h) { ri = i1; rj = j0 + t; slot = TY + t; }
-    else if ((t -= h) < w) { ri = i0 + t; rj = j0 - 1; slot = 2 * TY + t; }
-    else { t -= w; ri = i0 + t; rj = j1; slot = 2 * TY + TX + t; }
+    if (q < h) { ri = i0 - 1; rj = j0 + q; slot = q; }
+    else if ((q -= h) < h) { ri = i1; rj = j0 + q; slot = TY + q; }
+    else if ((q -= h) < w) { ri = i0 + q; rj = j0 - 1; slot = 2 * TY + q; }
+    else { q -= w; ri = i0 + q; rj = j1; slot = 2 * TY + f.wx + q; }
     return ri >= 0 && ri < nx && rj >= 0 && rj < ny;
   };
+  int my_ri = 0, my_rj = 0, my_slot = 0;
+  const bool my_ring = !comm && t < nring;
+  const bool my_in = my_ring && ring_cell(t, my_ri, my_rj, my_slot);
+  const int my_lp = lpad(my_ri, my_rj);
+  // RES: the mailbox, f.mail[parity][tile][slot]; nslot slots per tile (f.wx: the tile's width
+  // clipped to the grid's)
+  const int nslot = 2 * (TY + f.wx);
+  auto mailbox = [&](int parity, int q) -> ulonglong2* { return f.mail + ((size_t)parity * nb + q) * nslot; };
+  // w~ of a perimeter cell to the ring of every neighbour that reads it: first slots of the
+  // neighbours' rows (columns) that face this tile, -1 where there is no neighbour
+  const int slotW = bx > 0 ? (tile - 1) * nslot + TY : -1, slotE = i1 < nx ? (tile + 1) * nslot : -1;
+  const int slotS = by > 0 ? (tile - f.nbx) * nslot + 2 * TY + f.wx : -1;
+  const int slotN = j1 < ny ? (tile + f.nbx) * nslot + 2 * TY : -1;
+  const int hi_ = i1 - i0 - 1, hj_ = j1 - j0 - 1;  // last column and row
+  // (ir, jr): the cell within the tile
+  auto push = [&](int parity, unsigned int tag, int ir, int jr, double wk) {
+    ulonglong2* const m = mailbox(parity, 0);
+    if (ir == 0 && slotW >= 0) tag_put(m + slotW + jr, wk, tag);
+    if (ir == hi_ && slotE >= 0) tag_put(m + slotE + jr, wk, tag);
+    if (jr == 0 && slotS >= 0) tag_put(m + slotS + ir, wk, tag);
+    if (jr == hj_ && slotN >= 0) tag_put(m + slotN + ir, wk, tag);
+  };
+  const bool edge_col = tx == 0 || tx == hi_;
   const int8_t* __restrict__ kinds = a.kinds;
   const double* __restrict__ cus = a.cus;
   const double* __restrict__ cvs = a.cvs;
@@ -111,35 +169,33 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f) {
   const double ax = a.ax, ay = a.ay, dreg = a.dreg;
   double* __restrict__ xs = a.xs;
   double* __restrict__ p = a.p;
-  const KRow<double> K{a.cu, a.cv, a.dk, a.kind, a.creg_x, a.creg_y, a.dreg, (size_t)P};
+  auto sync_grid = [&]() -> bool { return range_sync(a.bar, a.bar.count, (unsigned int)nb, target); };
 
-  // r~ at neighbour (i, j) of an own cell after step 1: inside the tile from the next buffer,
-  // on the ring from shared memory
+  // r~ at neighbour (i, j) of an own cell after step 1 (without RES): inside the tile from the
+  // next buffer, on the ring from shared memory
   auto rnb = [&](const double* rn, int i, int j) -> double {
-    if constexpr (RES) return sr[lpad(i, j)];
     if (i < i0) return ring[j - j0];
     if (i >= i1) return ring[TY + (j - j0)];
     if (j < j0) return ring[2 * TY + (i - i0)];
-    if (j >= j1) return ring[2 * TY + TX + (i - i0)];
-    else return rn[g.idx(i, j)];
+    if (j >= j1) return ring[2 * TY + f.wx + (i - i0)];
+    return rn[g.idx(i, j)];
   };
-  // r~ of own cell (i, j) after step 1
-  auto rown = [&](const double* rn, int i, int j) -> double {
-    if constexpr (RES) return sr[lpad(i, j)];
-    else return rn[g.idx(i, j)];
-  };
-  // w~ of own cell (i, j) into the tile (RES, which also publishes the perimeter's r, w and s
-  // for iteration parity `pub`) or into wn
-  auto wput = [&](double* wn, int pub, int i, int j, double wk) {
+  // r~ of own cell (i, j) and its neighbours after step 1
+  auto gather = [&](const double* rn, int i, int j, double (&r)[5]) {
     if constexpr (RES) {
-      const int l = lidx(i, j);
+      const double* q = srn + lpad(i, j);
+      r[0] = q[0]; r[1] = q[-1]; r[2] = q[1]; r[3] = q[-TXP]; r[4] = q[TXP];
+    } else {
+      r[0] = rn[g.idx(i, j)];
+      r[1] = rnb(rn, i - 1, j); r[2] = rnb(rn, i + 1, j); r[3] = rnb(rn, i, j - 1); r[4] = rnb(rn, i, j + 1);
+    }
+  };
+  // w~ of own cell (i, j), tile-local index l, into the tile (RES, which also sends the
+  // perimeter's to the neighbours) or into wn
+  auto wput = [&](double* wn, int parity, unsigned int tag, int i, int j, int l, double wk) {
+    if constexpr (RES) {
       sw[l] = wk;
-      if (perimeter(i, j)) {
-        const size_t k = g.idx(i, j);
-        f.R[pub][k] = sr[lpad(i, j)];
-        f.W[pub][k] = wk;
-        f.S[pub][k] = ss[l];
-      }
+      if (i == i0 || i == i1 - 1 || j == j0 || j == j1 - 1) push(parity, tag, i - i0, j - j0, wk);
     } else {
       wn[g.idx(i, j)] = wk;
     }
@@ -147,207 +203,216 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f) {
   // Rows of cut cells and rows next to a Neumann side (kind 2) are listed per tile, in a fixed
   // order, at the start.  The stencil pass applies the constant stencil to every own cell, so
   // no warp diverges (an FP64 warp instruction costs the same however few of its lanes are
-  // active); a second pass, spread densely over the threads, corrects the listed cells.
+  // active); a second pass, spread densely over the threads, computes the listed cells.
   // Inactive cells (identity rows, kind 0) get their exact solution x = b in phase 0 and zero
-  // in every vector after it, so the stencil pass only has to write w = 0 there.  A tile with
-  // more listed cells than the list holds takes the general row for every cell instead.
-  int* const list = RES ? reinterpret_cast<int*>(skind + TXY) : reinterpret_cast<int*>(ring + 2 * (TX + TY));
-  double* const lcoef = reinterpret_cast<double*>(list + TXY);  // RES: 5 x kNT
-  __shared__ int s_scan[kNT / 32 + 1];
+  // in every vector after it.  A tile takes the general row for every cell instead where that is
+  // shorter: a warp then runs 8 FP64 operations per row instead of 6, and none of the 8 of each
+  // round of listed cells (a stretched mesh, every row of which has coefficients of its own; a
+  // small tile, of a few rows per thread, with any listed cell); and where the list does not hold
+  // them.  (The scaled coefficient arrays hold the constants on uniform rows and zeros on inactive
+  // ones.)
+  unsigned int m_in = 0u, m_list = 0u;  // RES: bit q: own cell q is inactive, is listed (nq <= 32)
   int nlist = 0;
-  bool general = false;
+  bool dense = false;
   {
     int mine = 0;
-    if (col)
-      for (int j = j0 + ty0; j < j1; j += RP) mine += kinds[g.idx(ci, j)] == 2;
+    for (int q = 0; q < nq; ++q) {
+      const int8_t km = kinds[k0 + q * kstep];
+      mine += km == 2;
+      if (RES) {
+        m_in |= (km == 0 ? 1u : 0u) << q;
+        m_list |= (km == 2 ? 1u : 0u) << q;
+      }
+    }
     // exclusive scan of the counts over the block (thread order)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
-    if (lane == 31) s_scan[wid] = incl;
+    if (!comm && lane == 31) sh.scan[wid] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       int acc = 0;
-      for (int q = 0; q < kNT / 32; ++q) {
-        const int c = s_scan[q];
-        s_scan[q] = acc;
+      for (int q = 0; q < NT / 32; ++q) {
+        const int c = sh.scan[q];
+        sh.scan[q] = acc;
         acc += c;
       }
-      s_scan[kNT / 32] = acc;
+      sh.scan[NT / 32] = acc;
+      sh.fail = 0;
     }
     __syncthreads();
-    nlist = s_scan[kNT / 32];
-    general = nlist > f.list_cap;
-    if (!general && mine > 0) {
-      int at = s_scan[wid] + incl - mine;
-      for (int j = j0 + ty0; j < j1; j += RP)
-        if (kinds[g.idx(ci, j)] == 2) list[at++] = (j - j0) * TX + tx;
+    nlist = sh.scan[NT / 32];
+    const int rows = (j1 - j0 + RP - 1) / RP;
+    dense = nlist > f.list_cap || 8 * rows < 6 * rows + 8 * ((nlist + NT - 1) / NT);
+    if (!dense && mine > 0) {
+      int at = sh.scan[wid] + incl - mine;
+      for (int q = 0; q < nq; ++q)
+        if (kinds[k0 + q * kstep] == 2) list[at++] = t + q * NT;
     }
     __syncthreads();
-    if constexpr (RES) {
-      // the first kNT listed cells' scaled coefficients, constant for the whole solve (listed
-      // cell q is taken by thread kNT - 1 - q, see below)
-      const int myq = kNT - 1 - (int)threadIdx.x;
-      if (f.lcache && !general && myq < nlist) {
-        const int q = list[myq];
-        const size_t k = g.idx(i0 + q % TX, j0 + q / TX);
-        lcoef[threadIdx.x] = cus[k];
-        lcoef[kNT + threadIdx.x] = cus[k + 1];
-        lcoef[2 * kNT + threadIdx.x] = cvs[k];
-        lcoef[3 * kNT + threadIdx.x] = cvs[k + P];
-        lcoef[4 * kNT + threadIdx.x] = sd[k];
-      }
-    }
   }
-  // Listed cell q is computed by thread kNT - 1 - q (then kNT - 1 - q + kNT, ...): threads are
+  // Listed cell q is computed by thread NT - 1 - q (then NT - 1 - q + NT, ...): threads are
   // ordered by the first row they take, so the last threads have the fewest own rows (with
   // TY = 27 and 4 rows per pass, the last 128 threads take 6 rows and the others 7), and a
   // tile's listed cells fill those free slots before they lengthen any warp.  An FP64-bound
   // sub-partition's time is the sum over its warps, and the slowest tile sets every
   // iteration's barrier.
-  const int myq = kNT - 1 - (int)threadIdx.x;
-  // the general row at own cell (i, j) (any kind); w = K~ r and the sums of a row of kind km
-  auto general_row = [&](const double* rn, int i, int j, double& rc_out) -> double {
-    const size_t k = g.idx(i, j);
+  const int myq = comm || dense ? nlist : NT - 1 - t;
+  int q_l = -1, q_i = 0, q_j = 0;  // this thread's first listed cell
+  if (myq < nlist) {
+    q_l = list[myq];
+    q_i = i0 + q_l % TX;
+    q_j = j0 + q_l / TX;
+  }
+  // The coefficients that the solve reads in every iteration, cached: W, E, S, N and d - dreg
+  auto coefs = [&](size_t k, double (&c)[5]) {
+    c[0] = cus[k]; c[1] = cus[k + 1]; c[2] = cvs[k]; c[3] = cvs[k + P];
     const int8_t km = kinds[k];
-    const double rc = rown(rn, i, j), rw = rnb(rn, i - 1, j), re = rnb(rn, i + 1, j);
-    const double rs = rnb(rn, i, j - 1), rq = rnb(rn, i, j + 1);
-    rc_out = rc;
-    if (km == 1) return rc - ax * (rw + re) - ay * (rs + rq);
-    if (km == 2) return rc - cus[k] * rw - cus[k + 1] * re - cvs[k] * rs - cvs[k + P] * rq;
-    return rc;
+    c[4] = (km == 1 ? dreg : (km == 2 ? sd[k] * sd[k] : 1.0)) - dreg;
   };
-  auto diag_of = [&](int i, int j) -> double {
-    const size_t k = g.idx(i, j);
-    const int8_t km = kinds[k];
-    return km == 1 ? dreg : (km == 2 ? sd[k] * sd[k] : 1.0);
+  if constexpr (RES) {
+    double c[5];
+    if (dense && f.dcache)
+      for (int q = 0, l = t; q < nq; ++q, l += NT) {
+        coefs(k0 + q * kstep, c);
+#pragma unroll
+        for (int e = 0; e < 5; ++e) dcoef[e * TXY + l] = c[e];
+      }
+    else if (f.lcache && q_l >= 0) {
+      coefs(g.idx(q_i, q_j), c);
+#pragma unroll
+      for (int e = 0; e < 5; ++e) lcoef[e * NT + t] = c[e];
+    }
+  }
+  // the general row: w = K~ r from r and its neighbours, and the sums
+  auto row = [&](const double (&r)[5], const double (&c)[5], double (&v)[4]) -> double {
+    const double wk = r[0] - c[0] * r[1] - c[1] * r[2] - c[2] * r[3] - c[3] * r[4];
+    const double r2 = r[0] * r[0];
+    v[0] += r2;
+    v[1] += c[4] * r2;
+    v[2] += wk * r[0];
+    return wk;
   };
   // step 2 on own cells: w = K~ r (r in buffer rn, or the tile with RES), sums into v
-  auto stencil = [&](const double* rn, double* wn, int pub, double (&v)[4]) {
-    if (general) {
-      if (col)
-        for (int j = j0 + ty0; j < j1; j += RP) {
-          double rc;
-          const double wk = general_row(rn, ci, j, rc);
-          wput(wn, pub, ci, j, wk);
-          v[0] += rc * rc;
-          v[1] += (diag_of(ci, j) - dreg) * (rc * rc);
-          v[2] += wk * rc;
+  auto stencil = [&](const double* rn, double* wn, int parity, unsigned int tag, double (&v)[4]) {
+    double r[5], c[5];
+    if (dense) {
+      for (int q = 0, l = t; q < nq; ++q, l += NT) {
+        const int j = j0 + ty0 + q * RP;
+        gather(rn, ci, j, r);
+        if (RES && f.dcache) {
+#pragma unroll
+          for (int e = 0; e < 5; ++e) c[e] = dcoef[e * TXY + l];
+        } else {
+          coefs(k0 + q * kstep, c);
         }
+        wput(wn, parity, tag, ci, j, l, row(r, c, v));
+      }
       return;
     }
-    // This thread's first listed cell: its values and coefficients are loaded before the
-    // constant-stencil pass, so that their latency overlaps it.
-    const int q0 = myq < nlist ? list[myq] : -1;
-    int li = 0, lj = 0;
-    double lr[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, lc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (q0 >= 0) {
-      li = i0 + q0 % TX;
-      lj = j0 + q0 / TX;
-      const size_t k = g.idx(li, lj);
-      lr[0] = rown(rn, li, lj); lr[1] = rnb(rn, li - 1, lj); lr[2] = rnb(rn, li + 1, lj);
-      lr[3] = rnb(rn, li, lj - 1); lr[4] = rnb(rn, li, lj + 1);
+    // the listed cells first: their chains of FP64 operations interleave with the other warps'
+    // constant-stencil passes instead of trailing them
+    if (q_l >= 0) {
+      gather(rn, q_i, q_j, r);
       if (RES && f.lcache) {
-        lc[0] = lcoef[threadIdx.x]; lc[1] = lcoef[kNT + threadIdx.x]; lc[2] = lcoef[2 * kNT + threadIdx.x];
-        lc[3] = lcoef[3 * kNT + threadIdx.x]; lc[4] = lcoef[4 * kNT + threadIdx.x];
+#pragma unroll
+        for (int e = 0; e < 5; ++e) c[e] = lcoef[e * NT + t];
       } else {
-        lc[0] = cus[k]; lc[1] = cus[k + 1]; lc[2] = cvs[k]; lc[3] = cvs[k + P]; lc[4] = sd[k];
+        coefs(g.idx(q_i, q_j), c);
+      }
+      wput(wn, parity, tag, q_i, q_j, q_l, row(r, c, v));
+    }
+    for (int q = myq + NT; q < nlist; q += NT) {
+      const int l = list[q], i = i0 + l % TX, j = j0 + l / TX;
+      gather(rn, i, j, r);
+      coefs(g.idx(i, j), c);
+      wput(wn, parity, tag, i, j, l, row(r, c, v));
+    }
+    // constant stencil on every own cell; the listed ones add nothing to the sums and are not
+    // stored (selects and predicates: a branch would run the FP64 instructions of both sides)
+    if constexpr (RES) {
+      const double* z = srn + lp0;
+#pragma unroll 2
+      for (int q = 0; q < nq; ++q, z += lpstep) {
+        const bool listed = (m_list >> q) & 1u;
+        const double rc = z[0];
+        double wk = rc - ax * (z[-1] + z[1]) - ay * (z[-TXP] + z[TXP]);
+        if ((m_in >> q) & 1u) wk = 0.0;
+        const double rs = listed ? 0.0 : rc;
+        v[0] += rs * rs;
+        v[2] += wk * rs;
+        if (!listed) {
+          sw[t + q * NT] = wk;
+          const int jr = ty0 + q * RP;
+          if (edge_col || jr == 0 || jr == hj_) push(parity, tag, tx, jr, wk);
+        }
+      }
+    } else {
+      for (int q = 0; q < nq; q += 2) {
+        const bool two = q + 1 < nq;
+        const int j = j0 + ty0 + q * RP, jb = two ? j + RP : j;
+        const size_t ka = k0 + q * kstep, kb = two ? ka + kstep : ka;
+        const int8_t kma = kinds[ka], kmb = kinds[kb];
+        double ra[5], rb[5];
+        gather(rn, ci, j, ra);
+        gather(rn, ci, jb, rb);
+        const double wa = kma == 0 ? 0.0 : ra[0] - ax * (ra[1] + ra[2]) - ay * (ra[3] + ra[4]);
+        if (kma != 2) {
+          wn[ka] = wa;
+          v[0] += ra[0] * ra[0];
+          v[2] += wa * ra[0];
+        }
+        if (two) {
+          const double wb = kmb == 0 ? 0.0 : rb[0] - ax * (rb[1] + rb[2]) - ay * (rb[3] + rb[4]);
+          if (kmb != 2) {
+            wn[kb] = wb;
+            v[0] += rb[0] * rb[0];
+            v[2] += wb * rb[0];
+          }
+        }
       }
     }
-    // constant stencil on every own cell but the listed ones, two rows of this thread at a time
-    if constexpr (RES) {
-      if (col)
-        for (int j = j0 + ty0; j < j1; j += RP) {
-          const int l = lidx(ci, j);
-          const int8_t km = skind[l];
-          const double rc = sr[lpad(ci, j)], rw = rnb(rn, ci - 1, j), re = rnb(rn, ci + 1, j);
-          const double rs = rnb(rn, ci, j - 1), rq = rnb(rn, ci, j + 1);
-          const double wk = km == 0 ? 0.0 : rc - ax * (rw + re) - ay * (rs + rq);
-          if (km != 2) {
-            wput(wn, pub, ci, j, wk);
-            v[0] += rc * rc;
-            v[2] += wk * rc;
-          }
-        }
-    } else {
-      if (col)
-        for (int j = j0 + ty0; j < j1; j += 2 * RP) {
-          const bool two = j + RP < j1;
-          const int jb = two ? j + RP : j;
-          const size_t ka = g.idx(ci, j), kb = g.idx(ci, jb);
-          const int8_t kma = kinds[ka], kmb = kinds[kb];
-          const double rca = rn[ka], rwa = rnb(rn, ci - 1, j), rea = rnb(rn, ci + 1, j);
-          const double rsa = rnb(rn, ci, j - 1), rqa = rnb(rn, ci, j + 1);
-          const double rcb = rn[kb], rwb = rnb(rn, ci - 1, jb), reb = rnb(rn, ci + 1, jb);
-          const double rsb = rnb(rn, ci, jb - 1), rqb = rnb(rn, ci, jb + 1);
-          const double wa = kma == 0 ? 0.0 : rca - ax * (rwa + rea) - ay * (rsa + rqa);
-          if (kma != 2) {
-            wn[ka] = wa;
-            v[0] += rca * rca;
-            v[2] += wa * rca;
-          }
-          if (two) {
-            const double wb = kmb == 0 ? 0.0 : rcb - ax * (rwb + reb) - ay * (rsb + rqb);
-            if (kmb != 2) {
-              wn[kb] = wb;
-              v[0] += rcb * rcb;
-              v[2] += wb * rcb;
-            }
-          }
-        }
-    }
-    // the listed cells: the general row
-    if (q0 >= 0) {
-      const double wk = lr[0] - lc[0] * lr[1] - lc[1] * lr[2] - lc[2] * lr[3] - lc[3] * lr[4];
-      wput(wn, pub, li, lj, wk);
-      v[0] += lr[0] * lr[0];
-      v[1] += (lc[4] * lc[4] - dreg) * (lr[0] * lr[0]);
-      v[2] += wk * lr[0];
-    }
-    for (int q = myq + kNT; q < nlist; q += kNT) {
-      const int loc = list[q];
-      const int i = i0 + loc % TX, j = j0 + loc / TX;
-      double rc;
-      const double wk = general_row(rn, i, j, rc);
-      wput(wn, pub, i, j, wk);
-      v[0] += rc * rc;
-      v[1] += (diag_of(i, j) - dreg) * (rc * rc);
-      v[2] += wk * rc;
-    }
   };
+  // FP64 sums of the computing threads' values over the block into rows[q * nb + tile] (all threads)
   auto reduce = [&](const double (&v)[4], int nv, double* rows) {
-    if (nv == 4) block_sum_warps<4, kNT>(v, red, bsum);
-    else {
-      const double v3[3] = {v[0], v[1], v[2]};
-      block_sum_warps<3, kNT>(v3, red, bsum);
+    if (!comm)
+      for (int q = 0; q < nv; ++q) sh.red[q][t] = v[q];
+    __syncthreads();
+    if (wid < nv) {
+      double s = 0.0;
+#pragma unroll
+      for (int m = 0; m < NT / 32; ++m) s += sh.red[wid][lane + 32 * m];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) sh.bsum[wid] = s;
     }
-    if (threadIdx.x == 0)
-      for (int q = 0; q < nv; ++q) rows[(size_t)q * nb + blockIdx.x] = bsum[q];
+    __syncthreads();
+    if (t == 0)
+      for (int q = 0; q < nv; ++q) rows[(size_t)q * nb + tile] = sh.bsum[q];
   };
   double* const rows0 = a.partials;              // reductions 0, 2, 4, ...
   double* const rows1 = a.partials + 4 * nb;     // reductions 1, 3, 5, ...
 
   // Phase 0: x~ = D^1/2 x, r_0 = D^-1/2 (b - K x) into R[0], s_{-1} = p_{-1} = 0.
   double v[4] = {0.0, 0.0, 0.0, 0.0};
-  if (col)
-    for (int j = j0 + ty0; j < j1; j += RP) {
-      const size_t k = g.idx(ci, j);
+  {
+    const KRow<double> K{a.cu, a.cv, a.dk, a.kind, a.creg_x, a.creg_y, a.dreg, (size_t)P};
+    for (int q = 0; q < nq; ++q) {
+      const size_t k = k0 + q * kstep;
       const double bk = a.b[k];
       const bool inactive = kinds[k] == 0;  // identity row: x = b exactly
       const double rk = inactive ? 0.0 : bk - K(a.x, k);
       const double x0 = inactive ? bk : sd[k] * a.x[k], r0 = a.isd[k] * rk;
-      if (RES) {
-        const int l = lidx(ci, j);
+      if constexpr (RES) {
+        const int l = t + q * NT, jr = ty0 + q * RP;
         sx[l] = x0;
-        sr[lpad(ci, j)] = r0;
+        srn[lp0 + q * lpstep] = r0;
         ss[l] = 0.0;
         sp[l] = 0.0;
-        skind[l] = kinds[k];
-        if (perimeter(ci, j)) f.R[0][k] = r0;  // the neighbours' first ring; S[0] and W[0] follow
+        if (edge_col || jr == 0 || jr == hj_) f.R[0][k] = r0;  // the neighbours' first ring
       } else {
         xs[k] = x0;
         f.R[0][k] = r0;
@@ -356,207 +421,319 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f) {
       }
       v[3] += bk * bk;
     }
-  // the fixed-point words start at zero (the previous launch leaves one buffer in use); the
+  }
+  // the fixed-point words and the mailboxes start at zero (they hold an earlier launch's); the
   // barriers of phase 0 order this before their first use
-  if (blockIdx.x == 0)
-    for (int q = threadIdx.x; q < 3 * kFxWords; q += kNT) f.fxacc[(size_t)q * kFxStride] = 0ULL;
-  bool ok = grid_sync(a.bar, target);
+  if (tile == 0 && t < 2 * kFxWords) f.fxacc[(size_t)t * kFxStride] = 0ULL;
+  if constexpr (RES)
+    for (int q = t; q < 2 * nslot; q += NT + 32)
+      mailbox(q >= nslot, tile)[q >= nslot ? q - nslot : q] = make_ulonglong2(0ULL, 0ULL);
+  bool ok = sync_grid();
   if (ok) {
     // w_0 = K~ r_0: every neighbour's r_0 is complete, read through the same ring path
-    for (int t = threadIdx.x; t < nring; t += kNT) {
-      int ri, rj, slot;
-      const bool in = ring_cell(t, ri, rj, slot);
-      const double rv0 = in ? f.R[0][g.idx(ri, rj)] : 0.0;
-      if constexpr (RES) sr[lpad(ri, rj)] = rv0;
-      else ring[slot] = rv0;
-    }
+    if (!comm)
+      for (int q = t; q < nring; q += NT) {
+        int ri, rj, slot;
+        const bool in = ring_cell(q, ri, rj, slot);
+        const double rv0 = in ? f.R[0][g.idx(ri, rj)] : 0.0;
+        if constexpr (RES) {
+          sr[lpad(ri, rj)] = srn[lpad(ri, rj)] = rv0;  // 0 outside the domain, in both frames, for good
+          ring[slot] = 0.0;                            // s_{-1}
+        } else {
+          ring[slot] = rv0;
+        }
+      }
     __syncthreads();
-    stencil(f.R[0], f.W[0], 0, v);
+    stencil(f.R[0], f.W[0], 0, 1u, v);
     reduce(v, 4, rows0);
-    ok = grid_sync(a.bar, target);
+    ok = sync_grid();
   }
-  int fx_lo = 0;  // bottom of the fixed-point window of the next reduction (same in every block)
+  // The communication warp's state: the recurrence, and its lanes' words after their last use
+  // (of the buffer next in turn and of the other).
+  CgState st{};
+  double thr = 0.0;  // tol^2 ||b||^2
+  double alpha = 0.0, beta = 0.0;
+  unsigned long long last = 0ULL, last2 = 0ULL;
+  int it = 0;
   if (ok) {
-    double t[4];
-    grid_sum<4>(rows0, nb, t, gsum);
-    if (threadIdx.x == 0) {
-      const double gamma = t[0], delta = t[2];
-      sc_rr = dreg * t[0] + t[1];
-      sc_bb = t[3];
-      sc_it = 0;
-      sc_stop = (sc_bb == 0.0 || sc_rr <= a.tol * a.tol * sc_bb) ? 1 : (a.max_iter <= 0 ? 2 : 0);
-      if (sc_stop == 0) {
-        sc_igamma = recip_newton(gamma);
-        sc_alpha = gamma * recip_newton(delta);
-        sc_den = delta;  // 1/alpha = den / gamma
-        sc_beta = 0.0;
+    double s[4];
+    grid_sum<4>(rows0, nb, s, sh.gsum);
+    if (comm) {
+      const double rr = dreg * s[0] + s[1];
+      const int stop = (s[3] == 0.0 || rr <= a.tol * a.tol * s[3]) ? 1 : (a.max_iter <= 0 ? 2 : 0);
+      const Scalar gamma = sc_of_double(s[0]);
+      st.igamma = cg_inverse(gamma);
+      st.den = sc_of_double(s[2]);
+      alpha = sc_double(sc_mul(gamma, sc_recip(st.den)));
+      thr = a.tol * a.tol * s[3];
+      if (lane == 0) {
+        sh.rr = rr;
+        sh.bb = s[3];
+        sh.stop = stop;
+        sh.alpha = alpha;
+        sh.beta = 0.0;
+        sh.lo = fx_window(s[0], s[1], s[2]);
       }
     }
     __syncthreads();
-    fx_lo = fx_window(t[0], t[1], t[2]);
   }
+  // The scalars of the next iteration from the sums of reduction `red` (1, 2, ...), in lane 0 of
+  // the communication warp: alpha and beta at once; then, while the other warps are in step 1
+  // with them, the stopping test and the window (step 1 leaves x~ alone, so an iteration that
+  // turns out to be one too many is dropped after it); 1 / gamma while they are in step 2.
+  auto scalars_rest = [&](const Scalar (&s)[3], int red) {
+    const double rr = dreg * sc_double(s[0]) + sc_double(s[1]);
+    sh.rr = rr;
+    sh.stop = rr <= thr ? 1 : (red >= a.max_iter ? 2 : 0);
+    sh.lo = max(max(sc_log2(s[0]), sc_log2(s[1])), sc_log2(s[2])) + kFxMargin - kFxTop;
+  };
   int cur = 0;
-  while (ok && sc_stop == 0) {
+  double my_w = 0.0;  // RES: w_i of this thread's first ring cell
+  if (RES && ok && sh.stop == 0 && my_in && !tag_wait(mailbox(0, tile) + my_slot, 1u, my_w, a.bar.budget, a.bar.err))
+    sh.fail = 1;  // seen behind the next block barrier
+  Scalar sums[3] = {};   // the last reduction's (communication warp)
+  long long digit = 0;   // and this lane's digit sum of it
+  bool rest = false;     // their stopping test is outstanding
+  while (ok) {
     const int nxt = cur ^ 1;
-    const double al = sc_alpha, be = sc_beta;
-    const double* __restrict__ rc_ = f.R[cur];
-    const double* __restrict__ wc_ = f.W[cur];
-    const double* __restrict__ sc_ = f.S[cur];
-    double* __restrict__ rn_ = f.R[nxt];
-    double* __restrict__ sn_ = f.S[nxt];
-    // this thread's first ring cell: the neighbours' iteration-i values, published before the
-    // last grid barrier, are loaded now so the L2 round trip overlaps step 1
-    int pf_slot = 0, pf_ri = 0, pf_rj = 0;
-    bool pf_in = false;
-    double pf_r = 0.0, pf_w = 0.0, pf_s = 0.0;
-    if (threadIdx.x < nring) {
-      int ri, rj;
-      pf_in = ring_cell(threadIdx.x, ri, rj, pf_slot);
-      pf_ri = ri;
-      pf_rj = rj;
-      if (pf_in) {
-        const size_t k = g.idx(ri, rj);
-        pf_r = rc_[k];
-        pf_w = wc_[k];
-        pf_s = sc_[k];
-      }
-    }
-    // step 1: own cells (RES: in the tile; otherwise two rows of this thread at a time with
-    // their loads in flight)
-    if (RES) {
-      if (col)
-        for (int j = j0 + ty0; j < j1; j += RP) {
-          const int l = lidx(ci, j);
-          const int lp = lpad(ci, j);
-          const double sk = sw[l] + be * ss[l], pk = sr[lp] + be * sp[l];
-          ss[l] = sk;
-          sp[l] = pk;
-          sr[lp] -= al * sk;
-        }
-    } else if (col)
-      for (int j = j0 + ty0; j < j1; j += 2 * RP) {
-        const bool two = j + RP < j1;
-        const size_t k0 = g.idx(ci, j), k1 = two ? g.idx(ci, j + RP) : k0;
-        const double r0 = rc_[k0], w0 = wc_[k0], s0 = sc_[k0], p0 = p[k0], x0 = xs[k0];
-        const double r1 = rc_[k1], w1 = wc_[k1], s1 = sc_[k1], p1 = p[k1], x1 = xs[k1];
-        {
-          const double sk = w0 + be * s0, pk = r0 + be * p0;
-          sn_[k0] = sk;
-          p[k0] = pk;
-          xs[k0] = x0 + al * pk;
-          rn_[k0] = r0 - al * sk;
-        }
-        if (two) {
-          const double sk = w1 + be * s1, pk = r1 + be * p1;
-          sn_[k1] = sk;
-          p[k1] = pk;
-          xs[k1] = x1 + al * pk;
-          rn_[k1] = r1 - al * sk;
-        }
-      }
-    // ring cells: r_{i+1} from the neighbours' iteration-i vectors
-    if (threadIdx.x < nring) {
-      const double rv0 = pf_in ? pf_r - al * (pf_w + be * pf_s) : 0.0;
-      if constexpr (RES) sr[lpad(pf_ri, pf_rj)] = rv0;
-      else ring[pf_slot] = rv0;
-    }
-    for (int t = threadIdx.x + kNT; t < nring; t += kNT) {
-      int ri, rj, slot;
-      double rv = 0.0;
-      if (ring_cell(t, ri, rj, slot)) {
-        const size_t k = g.idx(ri, rj);
-        rv = rc_[k] - al * (wc_[k] + be * sc_[k]);
-      }
-      if constexpr (RES) sr[lpad(ri, rj)] = rv;
-      else ring[slot] = rv;
-    }
-    __syncthreads();
-    v[0] = v[1] = v[2] = 0.0;
-    stencil(rn_, f.W[nxt], nxt, v);
-    // reduction sc_it + 1 in the rotating fixed-point buffers
-    const int ri = sc_it + 1, buf = ri % 3;
-    fx_arrive<kNT>(v, fx_lo, f.fxacc, buf, a.bar.absent, fxs);
-    if constexpr (RES) {
-      // x~ += alpha p_i is read by no other block and by nothing before the end: it runs between
-      // this block's arrival at the grid barrier and its wait
-      if (col)
-        for (int j = j0 + ty0; j < j1; j += RP) {
-          const int l = lidx(ci, j);
-          sx[l] += al * sp[l];
-        }
-    }
-    if (!fx_wait(f.fxacc, buf, (ri + 2) % 3, a.bar.budget, a.bar.err, fxs)) { ok = false; break; }
-    double t[3];
+    const int red = it + 1;                         // this iteration's reduction
+    const unsigned int tag = (unsigned int)it + 1u; // of w_i
+    const double al = sh.alpha, be = sh.beta;
     // every block takes the same branch: the overflow count is the grid's, and the test hook
     // depends on the reduction index only
-    const bool forced = f.fx_fallback_every > 0 && ri % f.fx_fallback_every == 0;
-    if (fxs.s[kFxWords - 1] == 0 && !forced) {
-      if (threadIdx.x < kFxQ) gsum[threadIdx.x] = fx_value(&fxs.s[threadIdx.x * kFxDigits], fx_lo);
-      __syncthreads();
-      t[0] = gsum[0];
-      t[1] = gsum[1];
-      t[2] = gsum[2];
-    } else {
-      // a value outside the window (every block sees the same count): this reduction again in
-      // FP64 through the partial rows and the counter barrier
-      double* const rows = (sc_it & 1) ? rows0 : rows1;
-      reduce(v, 3, rows);
-      if (!grid_sync(a.bar, target)) { ok = false; break; }
-      grid_sum<3>(rows, nb, t, gsum);
-    }
-    fx_lo = fx_window(t[0], t[1], t[2]);
-    // beta = gamma / gamma_old; alpha = gamma / (delta - beta gamma / alpha_old).  The two
-    // reciprocals are independent: 1/gamma (for the next beta) in warp 0, 1/den in warp 1,
-    // which issue to different sub-partitions' FP64 pipes.
-    if (threadIdx.x == 0) {
-      const double gamma = t[0];
-      sc_rr = dreg * t[0] + t[1];
-      sc_it += 1;
-      sc_stop = sc_rr <= a.tol * a.tol * sc_bb ? 1 : (sc_it >= a.max_iter ? 2 : 0);
-      if (sc_stop == 0) {
-        sc_beta = gamma * sc_igamma;
-        sc_igamma_next = recip_newton(gamma);
+    const bool forced = f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0;
+    if constexpr (RES) {
+      // the frame that received r_i becomes the current one
+      if (defer) {
+        double* const q = sr;
+        sr = srn;
+        srn = q;
       }
-    } else if (threadIdx.x == 32) {
-      const double gamma = t[0], delta = t[2];
-      const double beta = gamma * sc_igamma;
-      const double den = delta - beta * gamma * (sc_den * sc_igamma);
-      sc_den_next = den;
-      if (den != 0.0) sc_alpha = gamma * recip_newton(den);
+    }
+    v[0] = v[1] = v[2] = 0.0;
+    double* __restrict__ rn_ = f.R[nxt];
+    if (comm) {
+      if (rest && lane == 0) scalars_rest(sums, it);
+    } else {
+      const double* __restrict__ rc_ = f.R[cur];
+      const double* __restrict__ wc_ = f.W[cur];
+      const double* __restrict__ sc_ = f.S[cur];
+      double* __restrict__ sn_ = f.S[nxt];
+      double pf_r = 0.0, pf_w = 0.0, pf_s = 0.0;
+      if constexpr (!RES) {
+        // this thread's first ring cell: the neighbours' iteration-i values, published before the
+        // last reduction, are loaded now so the L2 round trip overlaps step 1
+        if (my_in) {
+          const size_t k = g.idx(my_ri, my_rj);
+          pf_r = rc_[k];
+          pf_w = wc_[k];
+          pf_s = sc_[k];
+        }
+      }
+      // step 1: own cells (RES: in the tile; otherwise two rows of this thread at a time with
+      // their loads in flight)
+      if constexpr (RES) {
+        if (defer) {
+#pragma unroll 2
+          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+            const double sk = sw[l] + be * ss[l];
+            ss[l] = sk;
+            srn[lp] = sr[lp] - al * sk;
+          }
+        } else {
+          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+            const double sk = sw[l] + be * ss[l], pk = sr[lp] + be * sp[l];
+            ss[l] = sk;
+            sp[l] = pk;
+            sr[lp] -= al * sk;
+          }
+        }
+      } else {
+        for (int q = 0; q < nq; q += 2) {
+          const bool two = q + 1 < nq;
+          const size_t ka = k0 + q * kstep, kb = two ? ka + kstep : ka;
+          const double r0 = rc_[ka], w0 = wc_[ka], s0 = sc_[ka];
+          const double r1 = rc_[kb], w1 = wc_[kb], s1 = sc_[kb];
+          const double ska = w0 + be * s0;
+          sn_[ka] = ska;
+          rn_[ka] = r0 - al * ska;
+          if (two) {
+            const double skb = w1 + be * s1;
+            sn_[kb] = skb;
+            rn_[kb] = r1 - al * skb;
+          }
+        }
+      }
+      // ring cells: r_{i+1} from the neighbours' iteration-i vectors; RES: w from the mailbox, r
+      // and s kept here (cells outside the domain stay 0)
+      if constexpr (RES) {
+        const ulonglong2* const box = mailbox(cur, tile);
+        auto ring_step = [&](int slot, int lp, double wv) {
+          const double sk = wv + be * ring[slot];
+          ring[slot] = sk;
+          srn[lp] = sr[lp] - al * sk;
+        };
+        if (my_in) ring_step(my_slot, my_lp, my_w);
+        for (int q = t + NT; q < nring; q += NT) {
+          int ri, rj, slot;
+          double wv = 0.0;
+          if (!ring_cell(q, ri, rj, slot)) continue;
+          if (!tag_wait(box + slot, tag, wv, a.bar.budget, a.bar.err)) sh.fail = 1;
+          ring_step(slot, lpad(ri, rj), wv);
+        }
+      } else {
+        if (my_ring) ring[my_slot] = my_in ? pf_r - al * (pf_w + be * pf_s) : 0.0;
+        for (int q = t + NT; q < nring; q += NT) {
+          int ri, rj, slot;
+          double rv = 0.0;
+          if (ring_cell(q, ri, rj, slot)) {
+            const size_t k = g.idx(ri, rj);
+            rv = rc_[k] - al * (wc_[k] + be * sc_[k]);
+          }
+          ring[slot] = rv;
+        }
+      }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      // read by warp 1 before the barrier above; next read after this iteration's barriers
-      sc_igamma = sc_igamma_next;
-      sc_den = sc_den_next;
+    if (sh.stop != 0 || sh.fail) break;
+    const int fx_lo = sh.lo;
+    if (!comm) {
+      stencil(rn_, f.W[nxt], nxt, tag + 1u, v);
+      fx_block_digits<NT>(v, fx_lo, sh.fx);
+      digits_ready<NT>(false);
+      if constexpr (RES) {
+        // the neighbours' w_{i+1} arrive about when their digits do: a first look now, its answer
+        // used after the update
+        ulonglong2* const box = mailbox(nxt, tile) + my_slot;
+        bool here = true;
+        if (my_in) here = tag_get(box, tag + 1u, my_w);
+        // read by no other block and by nothing before the end
+        if (defer) {
+#pragma unroll 2
+          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+            const double pk = sr[lp] + be * sp[l];
+            sp[l] = pk;
+            sx[l] += al * pk;
+          }
+        } else {
+          for (int q = 0, l = t; q < nq; ++q, l += NT) sx[l] += al * sp[l];
+        }
+        if (!here && !tag_wait(box, tag + 1u, my_w, a.bar.budget, a.bar.err)) sh.fail = 1;
+      } else {
+        const double* const rc_ = f.R[cur];
+        for (int q = 0; q < nq; q += 2) {
+          const size_t ka = k0 + q * kstep;
+          const bool two = q + 1 < nq;
+          const size_t kb = two ? ka + kstep : ka;
+          const double r0 = rc_[ka], p0 = p[ka], x0 = xs[ka], r1 = rc_[kb], p1 = p[kb], x1 = xs[kb];
+          const double pka = r0 + be * p0;
+          p[ka] = pka;
+          xs[ka] = x0 + al * pka;
+          if (two) {
+            const double pkb = r1 + be * p1;
+            p[kb] = pkb;
+            xs[kb] = x1 + al * pkb;
+          }
+        }
+      }
+    } else {
+      // The communication warp: arrive, wait, form the scalars.  Its code between the wait and the
+      // barrier is on every block's critical path and runs once per iteration, with cold
+      // instruction caches: so it runs twice, first on the previous reduction's digits while the
+      // digits of this one are still being formed.
+      if (rest && lane == 0) st.igamma = cg_inverse(sums[0]);
+      int over = 0;
+      bool got = true;
+      CgState next = st;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) {
+          digits_ready<NT>(true);
+          fx_arrive<NT, !RES>(f.fxacc, red & 1, tile == a.bar.absent, sh.fx);
+          got = fx_wait<!RES>(f.fxacc, red & 1, nb, a.bar.budget, a.bar.err, last, digit);
+        }
+        fx_sums(digit, fx_lo, sums, &over);
+        if (lane == 0) {
+          next = st;
+          cg_scalars(sums[0], sums[2], next, alpha, beta);
+          // (pass 0 writes what no one reads before pass 1 has written)
+          sh.alpha = alpha;
+          sh.beta = beta;
+        }
+      }
+      const unsigned long long q = last;
+      last = last2;
+      last2 = q;
+      rest = got && !forced && over == 0;
+      if (rest) st = next;
+      if (lane == 0) {
+        sh.redo = forced || over != 0;
+        if (!got) sh.fail = 1;
+      }
     }
+    __syncthreads();
+    if (sh.fail) { ok = false; break; }
+    if (sh.redo) {
+      // a value outside the window (every block sees the same count): this reduction again in
+      // FP64 through the partial rows and the counter barrier
+      double* const rows = (it & 1) ? rows0 : rows1;
+      reduce(v, 3, rows);
+      if (!sync_grid()) { ok = false; break; }
+      double d[3];
+      grid_sum<3>(rows, nb, d, sh.gsum);
+      if (comm) {
+        if (isfinite(d[0]) && isfinite(d[1]) && isfinite(d[2])) {
+#pragma unroll
+          for (int q = 0; q < 3; ++q) sums[q] = sc_of_double(d[q]);
+          if (lane == 0) {
+            cg_scalars(sums[0], sums[2], st, alpha, beta);
+            sh.alpha = alpha;
+            sh.beta = beta;
+          }
+          rest = true;
+        } else if (lane == 0) {
+          // not finite: nothing meets the tolerance any more
+          sh.alpha = sh.beta = sh.rr = d[0] + d[1] + d[2];
+          sh.stop = red >= a.max_iter ? 2 : 0;
+        }
+      }
+      __syncthreads();
+    }
+    it = red;
     cur = nxt;
   }
-  if (col)
-    for (int j = j0 + ty0; j < j1; j += RP) {
-      const size_t k = g.idx(ci, j);
-      a.x[k] = a.isd[k] * (RES ? sx[lidx(ci, j)] : xs[k]);
-    }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const bool conv = ok && sc_stop == 1;
-    a.out.iters[0] = ok ? sc_it : 0;
-    a.out.rr[0] = ok ? sc_rr : 0.0;
-    a.out.bb[0] = ok ? sc_bb : 0.0;
+  if (sh.fail) ok = false;
+  for (int q = 0; q < nq; ++q) {
+    const size_t k = k0 + q * kstep;
+    a.x[k] = a.isd[k] * (RES ? sx[t + q * NT] : xs[k]);
+  }
+  if (tile == 0 && t == 0) {
+    const bool conv = ok && sh.stop == 1;
+    a.out.iters[0] = ok ? it : 0;
+    a.out.rr[0] = ok ? sh.rr : 0.0;
+    a.out.bb[0] = ok ? sh.bb : 0.0;
     a.out.converged[0] = conv ? 1 : 0;
-    if (a.out.total && ok) a.out.total[0] += sc_it;
+    if (a.out.total && ok) a.out.total[0] += it;
     if (!conv && a.out.nconv) a.out.nconv[0] += 1;
   }
 }
 
-// __grid_constant__: the body takes the parameter by reference without a local copy
-__global__ void __launch_bounds__(kNT, 2) k_pcg_poisson_f1(const __grid_constant__ FusedSolve f) {
-  fused_body<false>(f);
+// __grid_constant__: the body takes the parameter by reference without a local copy.  MINB:
+// blocks per SM that must fit.
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f1(const __grid_constant__ FusedSolve f) {
+  __shared__ FusedShared<NT> sh;
+  fused_body<false, NT>(f, blockIdx.x, sh);
 }
-__global__ void __launch_bounds__(kNT, 2) k_pcg_poisson_f2(const __grid_constant__ FusedSolve f) {
-  fused_body<true>(f);
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f2(const __grid_constant__ FusedSolve f) {
+  __shared__ FusedShared<NT> sh;
+  fused_body<true, NT>(f, blockIdx.x, sh);
 }
 
 }  // namespace
+
+constexpr int kTileCells = 512;  // cells of a built-in plan's tile, at least about
 
 // Tile shape for at most `blocks` blocks: TX a power of two in 32..512, as many tile rows as
 // the blocks allow while a tile keeps about one cell per thread; the shape with the smallest
@@ -567,7 +744,7 @@ void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* nt
     const int bxn = (nx + tx - 1) / tx;
     if (bxn > blocks) continue;
     const int wx = std::min(tx, nx);
-    const int min_ty = (kNT + wx - 1) / wx;
+    const int min_ty = (kTileCells + wx - 1) / wx;
     const int byn = std::max(1, std::min(blocks / bxn, (ny + min_ty - 1) / min_ty));
     const int ty = (ny + byn - 1) / byn;
     const long long cells = (long long)wx * ty, ring = 2LL * (wx + ty);
@@ -582,75 +759,135 @@ void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* nt
   }
 }
 
-constexpr size_t kFusedSmemMax = 64 * 1024;  // ring and list of non-uniform cells, per block
+constexpr size_t kFusedSmemMax = 64 * 1024;  // f1: ring and list of non-uniform cells, per block
 
-int fused_blocks() {
-  int dev = 0, sms = 0, per = 0;
+namespace {
+
+int sm_count() {
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(k_pcg_poisson_f1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pcg_poisson_f1, kNT, kFusedSmemMax);
-  per = per > 2 ? 2 : (per < 1 ? 1 : per);
-  return sms * per;
+  return sms;
+}
+
+// Computing threads of a plan's blocks, the same whether its tiles are resident or not (so that
+// both run the same additions in the same order): one or two cells per thread on small tiles,
+// whose iteration is paced by its barriers and block sums; 512 where the FP64 pipe sets the pace;
+// 256 where two blocks of an SM share it (their threads then have registers enough).
+int fused_threads(int TX, int TY, int ntiles, int sms) {
+  const int cells = TX * TY;
+  if (cells <= 256 && TX <= 128) return 128;
+  if (TX <= 256 && (cells <= 1024 || (ntiles > sms && cells <= 2048))) return 256;
+  return 512;
+}
+
+const void* fused_kernel(bool resident, int nt, bool two) {
+  if (nt == 128) return resident ? (const void*)k_pcg_poisson_f2<128, 2> : (const void*)k_pcg_poisson_f1<128, 2>;
+  if (!resident) return nt == 256 ? (const void*)k_pcg_poisson_f1<256, 2> : (const void*)k_pcg_poisson_f1<512, 2>;
+  if (nt == 256) return two ? (const void*)k_pcg_poisson_f2<256, 2> : (const void*)k_pcg_poisson_f2<256, 1>;
+  return two ? (const void*)k_pcg_poisson_f2<512, 2> : (const void*)k_pcg_poisson_f2<512, 1>;
 }
 
 // Dynamic shared memory of a tile with its vectors resident (f2): x~, p, s, w, r~ with its
-// one-cell frame, the ring, the row kinds, a list of up to one entry per cell and, with `cache`,
-// the coefficients of kNT listed cells.
-size_t fused_resident_smem(int TX, int TY, bool cache) {
+// one-cell frame (two of them with `defer`), the ring's s, the coefficients of every cell
+// (`dcache`) or of nt listed cells (`lcache`), a list of up to one entry per cell.
+size_t resident_smem(int TX, int TY, int nt, bool dcache, bool defer, bool lcache) {
   const size_t txy = (size_t)TX * (size_t)TY;
-  return 4 * sizeof(double) * txy + sizeof(double) * ((size_t)TX + 2) * ((size_t)TY + 2) +
-         sizeof(double) * 2 * ((size_t)TX + (size_t)TY) + txy + sizeof(int) * txy +
-         (cache ? 5 * sizeof(double) * kNT : 0);
+  return sizeof(double) * (4 * txy + (defer ? 2 : 1) * ((size_t)TX + 2) * ((size_t)TY + 2) +
+                           2 * ((size_t)TX + (size_t)TY) + (dcache ? 5 * txy : 0) + (lcache ? 5 * (size_t)nt : 0)) +
+         sizeof(int) * txy;
 }
 
-// Whether ntiles tiles of TX x TY cells with resident vectors fit the GPU at once: with the
-// coefficient cache (2), only without it (1), or not at all (0).
-int fused_resident_fit(int TX, int TY, int ntiles) {
-  if (fused_resident_fits(TX, TY, ntiles, true)) return 2;
-  return fused_resident_fits(TX, TY, ntiles, false) ? 1 : 0;
-}
-bool fused_resident_ok(int TX, int TY, int ntiles) { return fused_resident_fit(TX, TY, ntiles) != 0; }
-
-bool fused_resident_fits(int TX, int TY, int ntiles, bool cache) {
-  const size_t smem = fused_resident_smem(TX, TY, cache);
-  int dev = 0, sms = 0, per = 0, optin = 0;
+// Shared memory of ntiles resident tiles of TX x TY cells, which must fit the GPU at once: with
+// every cell's coefficients cached, with a second r frame (defer) and with the listed cells'
+// coefficients cached where they fit too; 0 if nothing fits.
+size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
+  const int sms = sm_count(), nt = fused_threads(TX, TY, ntiles, sms);
+  if (ntiles < 1 || ntiles > 2 * sms || TX * TY > 32 * nt) return 0;
+  int dev = 0, optin = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (smem > (size_t)optin ||
-      cudaFuncSetAttribute(k_pcg_poisson_f2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pcg_poisson_f2, kNT, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  const void* kern = fused_kernel(true, nt, ntiles > sms);
+  for (int k = 7; k >= 0; --k) {
+    const bool dc = (k & 4) != 0, df = (k & 2) != 0, lc = (k & 1) != 0;
+    const size_t smem = resident_smem(TX, TY, nt, dc, df, lc);
+    if (smem > (size_t)optin) continue;
+    int per = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nt + 32, smem) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    if (ntiles > sms * std::min(per, 2)) continue;
+    if (f) {
+      f->dcache = dc ? 1 : 0;
+      f->defer = df ? 1 : 0;
+      f->lcache = lc ? 1 : 0;
+    }
+    return smem;
   }
-  return ntiles >= 1 && ntiles <= sms * std::min(per, 2);
+  return 0;
+}
+
+}  // namespace
+
+int fused_blocks() {
+  const void* kern = fused_kernel(false, 512, true);
+  int per = 0;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 512 + 32, kFusedSmemMax);
+  per = per > 2 ? 2 : (per < 1 ? 1 : per);
+  return sm_count() * per;
+}
+
+size_t fused_resident_smem_min(int TX, int TY) { return resident_smem(TX, TY, 0, false, false, false); }
+
+bool fused_resident_ok(int TX, int TY, int ntiles) { return resident_shape(TX, TY, ntiles, nullptr) != 0; }
+
+size_t fused_mail_slots(int nx, int TX, int TY, int ntiles) {
+  return (size_t)2 * (size_t)ntiles * 2 * (size_t)(TY + std::min(TX, nx));
+}
+
+// The most slots any resident plan of a grid can need: every tile width, every count of tile
+// rows up to kFusedTilesMax tiles whose smallest tile could stay in shared memory.
+size_t fused_mail_slots_max(int nx, int ny) {
+  size_t most = 0;
+  for (int tx = 32; tx <= 512; tx *= 2) {
+    const int bxn = (nx + tx - 1) / tx;
+    for (int byn = 1; byn <= ny && (long long)bxn * byn <= kFusedTilesMax; ++byn) {
+      const int ty = (ny + byn - 1) / byn;
+      if (fused_resident_smem_min(tx, ty) > 227 * 1024) continue;
+      most = std::max(most, fused_mail_slots(nx, tx, ty, bxn * ((ny + ty - 1) / ty)));
+    }
+  }
+  return most;
 }
 
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
-  const int blocks = fused_blocks();
+  const int blocks = fused_blocks(), sms = sm_count();
   if (f.TX == 0) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
   if (f.ntiles < 1) return cudaErrorInvalidConfiguration;
-  const void* kernel = (const void*)k_pcg_poisson_f1;
+  const int nt = fused_threads(f.TX, f.TY, f.ntiles, sms);
+  const void* kernel = fused_kernel(f.resident != 0, nt, f.ntiles > sms);
   size_t smem = 0;
+  f.wx = std::min(f.TX, f.a.g.nx);
   if (f.resident) {
     // the tile's vectors in shared memory: as many blocks as fit must hold every tile
-    const int fit = fused_resident_fit(f.TX, f.TY, f.ntiles);
-    if (fit == 0) return cudaErrorInvalidConfiguration;
-    f.lcache = fit == 2 ? 1 : 0;
-    smem = fused_resident_smem(f.TX, f.TY, f.lcache != 0);
+    smem = resident_shape(f.TX, f.TY, f.ntiles, &f);
+    if (smem == 0 || !f.mail || f.mail_slots < fused_mail_slots(f.a.g.nx, f.TX, f.TY, f.ntiles))
+      return cudaErrorInvalidConfiguration;
     f.list_cap = f.TX * f.TY;
-    kernel = (const void*)k_pcg_poisson_f2;
   } else {
     const size_t ring = sizeof(double) * 2 * ((size_t)f.TX + (size_t)f.TY);
     if (ring + sizeof(int) * 256 > kFusedSmemMax || f.ntiles > blocks) return cudaErrorInvalidConfiguration;
     // the list of non-uniform cells takes what is left, up to one entry per tile cell
     f.list_cap = (int)std::min<size_t>((kFusedSmemMax - ring) / sizeof(int), (size_t)f.TX * (size_t)f.TY);
     smem = ring + sizeof(int) * (size_t)f.list_cap;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
   }
   cudaMemsetAsync(f.a.bar.count, 0, sizeof(unsigned int) * kBarWords, st);
   void* params[] = {&f};
-  return cudaLaunchCooperativeKernel(kernel, f.ntiles, kNT, params, smem, st);
+  return cudaLaunchCooperativeKernel(kernel, f.ntiles, nt + 32, params, smem, st);
 }
 
 }  // namespace ccm
