@@ -298,9 +298,16 @@ void set_uniform_coefficients(ccm_case c, PoissonSolve<T>& a) {
 }
 
 ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
-  if (!c->zero_mean && c->cfg.precond == CCM_JACOBI && !c->g.px && !c->g.py) {
-    // Jacobi-PCG as CG on the symmetrically scaled system (nonsingular systems)
-    // with one grid barrier per iteration (tiles that recompute their ring)
+  if (c->cfg.precond == CCM_JACOBI && !c->g.px && !c->g.py) {
+    // Jacobi-PCG as CG on the symmetrically scaled system with one grid barrier per iteration
+    // (tiles that recompute their ring).  A singular system takes the same iteration: with a
+    // zero-mean right-hand side its residuals stay orthogonal to the null space (the constants),
+    // so alpha, beta and r are those of the iteration that projects every preconditioned residual,
+    // and the iterates differ from its by a constant, which the last projection removes.
+    if (c->zero_mean) {
+      CUDA_TRY(project_zero_mean(c->g, c->co.act, x, c->partials, c->n_act, c->st));
+      CUDA_TRY(project_zero_mean(c->g, c->co.act, b, c->partials, c->n_act, c->st));
+    }
     CaseSolveView v;
     case_solve_view(c, &v);
     FusedSolve f{};
@@ -315,7 +322,7 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
     f.R[0] = c->pr; f.R[1] = c->pz2;
     f.W[0] = c->pq; f.W[1] = c->pw1;
     f.S[0] = c->pp1; f.S[1] = c->t5;
-    if (c->tune.cluster > 0) {
+    if (c->tune.cluster > 0 && !c->zero_mean) {
       // small grid: the whole solve inside one thread-block cluster
       ClusterSolve cs{};
       cs.a = f.a;
@@ -325,6 +332,7 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
     const TilePlan& tp = c->tune.plan;
     f.TX = tp.TX; f.TY = tp.TY; f.nbx = tp.nbx; f.ntiles = tp.ntiles; f.resident = tp.resident;
     CUDA_TRY(run_poisson_fused(f, c->st));
+    if (c->zero_mean) CUDA_TRY(project_zero_mean(c->g, c->co.act, x, c->partials, c->n_act, c->st));
     return CCM_OK;
   }
   PoissonSolve<double> a{};
@@ -597,7 +605,7 @@ ccm_status poisson_solve(ccm_case c, double* x, double* b) {
   ccm_status s = solve_poisson_fp64(c, x, b);
   if (c->timing && e1) cudaEventRecord(e1, c->st);
   c->poisson_launches++;
-  c->launches += c->zero_mean ? 5 : 1;
+  c->launches += c->zero_mean ? (c->cfg.precond == CCM_JACOBI && !c->g.px && !c->g.py ? 7 : 5) : 1;
   launch_wrap_cells(c->g, x, c->st);  // periodic sides: Phi's images for the projection
   return s;
 }

@@ -112,7 +112,7 @@ struct FusedSolve {
   double* S[2];
   ulonglong2* mail;         // resident tiles: mailboxes, mail_slots 16-byte slots (cleared by the kernel itself)
   size_t mail_slots;
-  int TX, TY, nbx, ntiles;  // tile plan; TX = 0 lets the launcher choose
+  int TX, TY, nbx, ntiles;  // tile plan; TX = 0 lets the launcher choose (resident where that fits)
   int resident;             // 1: each tile keeps its vectors in shared memory (k_pcg_poisson_f2)
   // set by the launcher
   int wx;                   // TX clipped to the grid's width
@@ -123,7 +123,7 @@ struct FusedSolve {
 };
 constexpr int kFusedTilesMax = 512;  // tiles of a launch, at most (two per SM)
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles);
+void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells = 512);
 int fused_blocks();
 size_t fused_resident_smem_min(int TX, int TY);
 bool fused_resident_ok(int TX, int TY, int ntiles);

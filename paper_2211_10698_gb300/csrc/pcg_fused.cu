@@ -733,18 +733,16 @@ __global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f2(const __grid_c
 
 }  // namespace
 
-constexpr int kTileCells = 512;  // cells of a built-in plan's tile, at least about
-
 // Tile shape for at most `blocks` blocks: TX a power of two in 32..512, as many tile rows as
-// the blocks allow while a tile keeps about one cell per thread; the shape with the smallest
+// the blocks allow while a tile keeps about min_cells cells; the shape with the smallest
 // largest tile wins (then the shortest ring).  One block per tile.
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles) {
+void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells) {
   long long best = -1, best_ring = 0;
   for (int tx = 32; tx <= 512; tx *= 2) {
     const int bxn = (nx + tx - 1) / tx;
     if (bxn > blocks) continue;
     const int wx = std::min(tx, nx);
-    const int min_ty = (kTileCells + wx - 1) / wx;
+    const int min_ty = (min_cells + wx - 1) / wx;
     const int byn = std::max(1, std::min(blocks / bxn, (ny + min_ty - 1) / min_ty));
     const int ty = (ny + byn - 1) / byn;
     const long long cells = (long long)wx * ty, ring = 2LL * (wx + ty);
@@ -863,9 +861,18 @@ size_t fused_mail_slots_max(int nx, int ny) {
   return most;
 }
 
+// Cells of a built-in resident tile, at least about.
+constexpr int kResidentCells = 128;
+
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   const int blocks = fused_blocks(), sms = sm_count();
-  if (f.TX == 0) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
+  if (f.TX == 0) {
+    // the built-in plan: resident tiles, one per SM, where they fit, else two in global memory
+    fused_tiles(f.a.g.nx, f.a.g.ny, sms, &f.TX, &f.TY, &f.nbx, &f.ntiles, kResidentCells);
+    f.resident = resident_shape(f.TX, f.TY, f.ntiles, nullptr) != 0 && f.mail &&
+                 f.mail_slots >= fused_mail_slots(f.a.g.nx, f.TX, f.TY, f.ntiles);
+    if (!f.resident) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
+  }
   if (f.ntiles < 1) return cudaErrorInvalidConfiguration;
   const int nt = fused_threads(f.TX, f.TY, f.ntiles, sms);
   const void* kernel = fused_kernel(f.resident != 0, nt, f.ntiles > sms);
