@@ -92,7 +92,6 @@ struct ScaledSolve {
   Barrier bar;
   PcgOut out;
 };
-cudaError_t run_poisson_scaled(const ScaledSolve& a, cudaStream_t st);
 
 // The same solve with one grid barrier per iteration (pcg_fused.cu): 2-D tiles, the ring of
 // each tile recomputed by its block, r, w, s double-buffered.  a.xs and a.p are used, a.r,

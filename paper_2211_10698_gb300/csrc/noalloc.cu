@@ -6,13 +6,12 @@
 // synchronisation that cudaMalloc and cudaFree imply.  ccm_solve_pressure_noalloc serves
 // them: it solves the same system as ccm_solve_pressure in FP64 with the Jacobi
 // preconditioner, whatever the case's precision and preconditioner settings, but its scratch
-// vectors live in one file-scope __device__ array of fixed size instead of memory the
-// library allocates.  Two kernels serve it: a case with an outflow side and the Jacobi
-// setting runs CG on the Jacobi-scaled system in the two-barrier layout (k_pcg_poisson_sc,
-// which needs fewer work vectors than the tiled one); a singular case (no outflow side,
-// zero-mean iterates) or one configured for Chebyshev runs the unscaled Jacobi-PCG
-// (k_pcg_poisson_cg with a degree-1 preconditioner).  The caller passes the right-hand side
-// and the solution in device memory of its own.
+// lives in one file-scope __device__ array of fixed size instead of memory the library
+// allocates.  The kernel is the resident one-barrier solve (pcg_fused.cu) in its built-in plan:
+// a tile's vectors stay in shared memory, so the array holds the right-hand side, the first
+// residual and the mailboxes of the tiles (every grid within the limit fits: at most 863 cells
+// per SM).  A singular case (no outflow side) projects onto zero mean at the start and the end.
+// The caller passes the right-hand side and the solution in device memory of its own.
 //
 // The array (about 6.4 MB) stays resident on every GPU that loads the library until the
 // process exits.  Every call uses the same array, so calls that overlap on the GPU (from
@@ -37,13 +36,11 @@ constexpr size_t kMaxPartials = 8192;
 constexpr int kMaxDevices = 64;
 
 struct Scratch {
-  double b[kMaxElems];  // right-hand side restricted to active cells
-  double r[kMaxElems];
-  double u[kMaxElems];
-  double w[kMaxElems];
-  double p[kMaxElems];
-  double s[kMaxElems];
+  double b[kMaxElems];           // right-hand side restricted to active cells
+  double r[kMaxElems];           // the tiles' first residual
+  ulonglong2 mail[2 * kMaxElems];  // the tiles' mailboxes
   double partials[kMaxPartials];
+  unsigned long long fxacc[kFxAccWords];
   double rr, bb;
   int iters, converged;
   int bar_err, pad;
@@ -111,43 +108,30 @@ extern "C" ccm_status ccm_solve_pressure_noalloc(ccm_case c, const double* rhs_d
   cudaError_t e = scratch_address(&S);
   if (e != cudaSuccess) return fail(CCM_E_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
   cudaStream_t st = v.st;
-  // the previous call's contents (possibly of another grid size): the first n elements of
-  // every work vector are cleared, since the stencils read them on the ghost ring (a solve
-  // of this grid touches nothing beyond them), and so are the barrier counter and its
-  // error flag
-  double* const work[5] = {S->r, S->u, S->w, S->p, S->s};
-  for (double* a : work)
-    if ((e = cudaMemsetAsync(a, 0, n * sizeof(double), st)) != cudaSuccess)
-      return fail(CCM_E_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+  // the barrier counter and its error flag hold the previous call's (the kernel clears or writes
+  // the rest of the scratch before it reads it)
   if ((e = cudaMemsetAsync(&S->bar_err, 0, 2 * sizeof(int) + sizeof(unsigned int) * kBarWords, st)) != cudaSuccess)
     return fail(CCM_E_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   const dim3 blk(64, 4), grd((v.g.nx + 3 + 63) / 64, (v.g.ny + 3 + 3) / 4);
   k_masked_copy<<<grd, blk, 0, st>>>(v.g, v.act, rhs_dev, S->b);
   k_mask<<<grd, blk, 0, st>>>(v.g, v.act, phi_dev);
-  if (!v.zero_mean && v.precond == CCM_JACOBI) {
-    ScaledSolve q = scaled_solve_of(v, phi_dev, S->b, S->u, S->r, S->w, S->p, S->s);
-    q.partials = S->partials;
-    q.bar = Barrier{S->bar_count, &S->bar_err, 2000000000LL};
-    q.out = PcgOut{&S->iters, &S->rr, &S->bb, &S->converged, nullptr, nullptr};
-    e = run_poisson_scaled(q, st);
-  } else {
-    PoissonSolve<double> a{};
-    a.g = v.g;
-    a.cu = v.cu; a.cv = v.cv; a.dk = v.dk; a.invd = v.invd; a.kind = v.kind;
-    a.creg_x = v.g.hy / v.g.hx;
-    a.creg_y = v.g.hx / v.g.hy;
-    a.dreg = 2.0 * (a.creg_x + a.creg_y);
-    a.invd_reg = 1.0 / a.dreg;
-    a.x = phi_dev; a.b = S->b; a.r = S->r; a.z = S->u; a.q = S->w; a.p0 = S->p; a.p1 = S->s;
-    a.z2 = nullptr; a.w1 = nullptr;
-    a.cheb = 1;
-    a.tol = v.tol; a.max_iter = v.max_iter;
-    a.zero_mean = v.zero_mean; a.n_act = v.n_act;
-    a.partials = S->partials;
-    a.bar = Barrier{S->bar_count, &S->bar_err, 2000000000LL};
-    a.out = PcgOut{&S->iters, &S->rr, &S->bb, &S->converged, nullptr, nullptr};
-    e = run_poisson_pcg<double>(a, st);
+  FusedSolve f{};
+  f.a = scaled_solve_of(v, phi_dev, S->b, nullptr, nullptr, nullptr, nullptr, nullptr);
+  f.a.partials = S->partials;
+  f.a.bar = Barrier{S->bar_count, &S->bar_err, 2000000000LL};
+  f.a.out = PcgOut{&S->iters, &S->rr, &S->bb, &S->converged, nullptr, nullptr};
+  f.fxacc = S->fxacc;
+  f.R[0] = S->r;
+  f.mail = S->mail;
+  f.mail_slots = 2 * kMaxElems;
+  f.resident = 1;
+  e = cudaSuccess;
+  if (v.zero_mean) {
+    e = project_zero_mean(v.g, v.act, phi_dev, S->partials, v.n_act, st);
+    if (e == cudaSuccess) e = project_zero_mean(v.g, v.act, S->b, S->partials, v.n_act, st);
   }
+  if (e == cudaSuccess) e = run_poisson_fused(f, st);
+  if (e == cudaSuccess && v.zero_mean) e = project_zero_mean(v.g, v.act, phi_dev, S->partials, v.n_act, st);
   if (e != cudaSuccess)
     return fail(CCM_E_CUDA, std::string("Poisson PCG launch: ") + cudaGetErrorString(e));
   struct { double rr, bb; int iters, converged; int err, pad; } h{};

@@ -1,5 +1,5 @@
 // FP64 pressure Poisson solve (Eq. pm_poisson) for small grids: CG on the Jacobi-scaled system
-// (the iteration of pcg_scaled.cu) inside ONE thread-block cluster.
+// (the system of pcg_scaled.cu) inside ONE thread-block cluster.
 //
 // On a grid of a few thousand cells a grid-wide barrier and the L2 round trips of each phase
 // cost several times the arithmetic.  Here the C CTAs of one cluster (C <= 16, one per SM)
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kCT, 1) k_pcg_poisson_cluster(ClusterSolve f) 
   const KRow<double> K{a.cu, a.cv, a.dk, a.kind, a.creg_x, a.creg_y, a.dreg, (size_t)P};
   const double ax = a.ax, ay = a.ay, dreg = a.dreg;
 
-  // B: w = K~ r on the band and the sums (as in pcg_scaled.cu); neighbours outside the domain
+  // B: w = K~ r on the band and the sums (as in pcg_fused.cu); neighbours outside the domain
   // are zero (the scaled coefficients of faces to ghost cells are zero too)
   auto phase_b = [&](double (&v)[4]) {
     for (int l = threadIdx.x; l < ncell; l += kCT) {

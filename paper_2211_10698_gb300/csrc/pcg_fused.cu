@@ -1,7 +1,7 @@
-// FP64 pressure Poisson solve (Eq. pm_poisson) by CG on the Jacobi-scaled system (the
-// iteration of pcg_scaled.cu) with ONE grid barrier per iteration.
+// FP64 pressure Poisson solve (Eq. pm_poisson) by CG on the Jacobi-scaled system (pcg_scaled.cu)
+// with ONE grid barrier per iteration.
 //
-// In pcg_scaled.cu an iteration needs two device-wide barriers: one so that the stencil
+// Plainly, an iteration needs two device-wide barriers: one so that the stencil
 // w = K~ r sees the neighbours' new residual, one for the dot products.  Here each block
 // owns a 2-D tile of cells and computes the new residual of the one-cell ring around its tile
 // itself, from the previous iteration's vectors:
@@ -869,9 +869,11 @@ cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   if (f.TX == 0) {
     // the built-in plan: resident tiles, one per SM, where they fit, else two in global memory
     fused_tiles(f.a.g.nx, f.a.g.ny, sms, &f.TX, &f.TY, &f.nbx, &f.ntiles, kResidentCells);
-    f.resident = resident_shape(f.TX, f.TY, f.ntiles, nullptr) != 0 && f.mail &&
-                 f.mail_slots >= fused_mail_slots(f.a.g.nx, f.TX, f.TY, f.ntiles);
-    if (!f.resident) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
+    const bool fits = resident_shape(f.TX, f.TY, f.ntiles, nullptr) != 0 && f.mail &&
+                      f.mail_slots >= fused_mail_slots(f.a.g.nx, f.TX, f.TY, f.ntiles);
+    if (!fits && f.resident) return cudaErrorInvalidConfiguration;  // the caller has resident tiles only
+    if (!fits) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
+    f.resident = fits ? 1 : 0;
   }
   if (f.ntiles < 1) return cudaErrorInvalidConfiguration;
   const int nt = fused_threads(f.TX, f.TY, f.ntiles, sms);

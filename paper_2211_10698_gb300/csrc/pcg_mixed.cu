@@ -4,7 +4,7 @@
 // solvers by Clark et al., Comput. Phys. Commun. 181, 2010).
 //
 // The iterate x and the right-hand side b stay in FP64.  Between replacements the kernel runs
-// the single-reduction CG of pcg_scaled.cu in FP32 on the correction equation
+// the single-reduction CG on the system of pcg_scaled.cu in FP32 on the correction equation
 //     K~ e~ = r~,   r~ = sigma D^-1/2 (b - K x),
 // normalised by sigma = 1 / ||D^-1/2 (b - K x)|| so the FP32 values stay near unit size
 // whatever the scale of b.  When the FP32 residual has dropped by the factor `drop` since the
