@@ -297,6 +297,22 @@ void set_uniform_coefficients(ccm_case c, PoissonSolve<T>& a) {
   a.invd_reg = 1.0 / a.dreg;
 }
 
+// The one-barrier FP64 solve of a case (x = solution in/out, b = right-hand side) on its work arrays;
+// partials, bar, out and the tile plan are the caller's.
+FusedSolve fused_solve_of(ccm_case c, double* x, const double* b) {
+  CaseSolveView v;
+  case_solve_view(c, &v);
+  FusedSolve f{};
+  f.a = scaled_solve_of(v, x, b, c->pz, nullptr, nullptr, c->pp0, nullptr);
+  f.fxacc = c->fxacc;
+  f.mail = c->mail;
+  f.mail_slots = c->mail_slots;
+  f.R[0] = c->pr; f.R[1] = c->pz2;
+  f.W[0] = c->pq; f.W[1] = c->pw1;
+  f.S[0] = c->pp1; f.S[1] = c->t5;
+  return f;
+}
+
 ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
   if (c->cfg.precond == CCM_JACOBI && !c->g.px && !c->g.py) {
     // Jacobi-PCG as CG on the symmetrically scaled system with one grid barrier per iteration
@@ -308,20 +324,11 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
       CUDA_TRY(project_zero_mean(c->g, c->co.act, x, c->partials, c->n_act, c->st));
       CUDA_TRY(project_zero_mean(c->g, c->co.act, b, c->partials, c->n_act, c->st));
     }
-    CaseSolveView v;
-    case_solve_view(c, &v);
-    FusedSolve f{};
-    f.a = scaled_solve_of(v, x, b, c->pz, nullptr, nullptr, c->pp0, nullptr);
-    f.fxacc = c->fxacc;
-    f.mail = c->mail;
-    f.mail_slots = c->mail_slots;
+    FusedSolve f = fused_solve_of(c, x, b);
     f.fx_fallback_every = c->fx_fallback_every;
     f.a.partials = c->partials;
     f.a.bar = case_barrier(c);
     f.a.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, &c->ds->total_p, &c->ds->nconv};
-    f.R[0] = c->pr; f.R[1] = c->pz2;
-    f.W[0] = c->pq; f.W[1] = c->pw1;
-    f.S[0] = c->pp1; f.S[1] = c->t5;
     if (c->tune.cluster > 0 && !c->zero_mean) {
       // small grid: the whole solve inside one thread-block cluster
       ClusterSolve cs{};
@@ -539,21 +546,12 @@ ccm_status autotune_poisson(ccm_case c) {
     const std::vector<TilePlan> cand = fused_plan_candidates(g.nx, g.ny, most);
     const std::vector<int> ccand = cluster_candidates(g.nx, g.ny);
     const int nf = (int)cand.size();
-    CaseSolveView v;
-    case_solve_view(c, &v);
-    FusedSolve f{};
-    f.a = scaled_solve_of(v, x, b, c->pz, nullptr, nullptr, c->pp0, nullptr);
-    f.fxacc = c->fxacc;
-    f.mail = c->mail;
-    f.mail_slots = c->mail_slots;
+    FusedSolve f = fused_solve_of(c, x, b);
     f.a.partials = c->partials;
     f.a.bar = case_barrier(c);
     f.a.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, nullptr, nullptr};
     f.a.tol = 0.0;
     f.a.max_iter = kTuneIters;
-    f.R[0] = c->pr; f.R[1] = c->pz2;
-    f.W[0] = c->pq; f.W[1] = c->pw1;
-    f.S[0] = c->pp1; f.S[1] = c->t5;
     e = time_launches(nf + (int)ccand.size(), [&](int k) -> cudaError_t {
       cudaError_t me = cudaMemsetAsync(x, 0, bytes, st);
       if (me != cudaSuccess) return me;
@@ -715,6 +713,11 @@ void case_scaled_fp64(ccm_case c, ScaledSolve* a) {
   case_solve_view(c, &v);
   *a = scaled_solve_of(v, c->phi, c->rhs_p, c->pz, c->pr, c->pq, c->pp0, c->pp1);
   a->out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, &c->ds->total_p, &c->ds->nconv};
+}
+void case_fused_fp64(ccm_case c, FusedSolve* f) {
+  *f = fused_solve_of(c, c->phi, c->rhs_p);
+  f->a.partials = c->partials;
+  f->a.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, &c->ds->total_p, &c->ds->nconv};
 }
 void case_mixed_batch(ccm_case c, MixedSolve* a) { case_mixed_solve(c, c->phi, c->rhs_p, a); }
 

@@ -6,8 +6,9 @@
 // (operators.cu), the CN Helmholtz solves one cooperative launch (pcg_helm.cu), and the
 // pressure Poisson solves one cooperative launch (each case gets a contiguous range of blocks
 // in proportion to its expected work and reduces over its own blocks).  When every case has
-// an outflow side (nonsingular systems) the Poisson launch is k_sc_batch (FP64 CG on the
-// Jacobi-scaled systems) or k_mixed_batch (FP32 CG with FP64 residual replacements, Jacobi or
+// an outflow side (nonsingular systems) the Poisson launch is k_fused_batch (FP64 CG on the
+// Jacobi-scaled systems, every tile's vectors resident in shared memory; pcg_fused.cu) where the
+// cases' tiles fit the GPU at once, else k_sc_batch (vectors in global memory), or k_mixed_batch (FP32 CG with FP64 residual replacements, Jacobi or
 // Chebyshev per case, for the MIXED setting), both in pcg_batch.cu.  Otherwise the unscaled
 // Jacobi-PCG batch of pcg.cu runs, and for MIXED the FP64 residual refinement runs from the
 // host for the whole batch: residuals of the unconverged cases, one host check, one batched
@@ -31,6 +32,10 @@ struct ccm_batch_s {
   BatchEntry<double>* e64 = nullptr;
   BatchEntry<float>* e32 = nullptr;
   ScaledBatchEntry* esc = nullptr;
+  FusedBatchEntry* efu = nullptr;
+  bool fused = false;            // the FP64 tables on the device are efu's (resident tiles)
+  int fused_nblocks = 0;
+  size_t fused_smem = 0;
   MixedBatchEntry* emx = nullptr;
   int* block_case = nullptr;
   double* partials = nullptr;
@@ -80,12 +85,17 @@ ccm_status bfail(ccm_status s, const std::string& m) {
 // Contiguous block ranges for the cases' expected work w: at least one block per case, then
 // each further block to the case whose work per block is largest (this minimises the largest
 // work per block, which sets the launch's length: every slot waits for the slowest block).
-void allocate_blocks(const std::vector<double>& w, int blocks, std::vector<int>& b0, std::vector<int>& nb) {
+// least (may be null): blocks that each case needs at least.
+void allocate_blocks(const std::vector<double>& w, int blocks, std::vector<int>& b0, std::vector<int>& nb,
+                     const std::vector<int>* least = nullptr) {
   const int n = (int)w.size();
   nb.assign(n, 1);
+  if (least) nb = *least;
+  int left = blocks;
+  for (int k : nb) left -= k;
   std::priority_queue<std::pair<double, int>> q;
-  for (int i = 0; i < n; ++i) q.push({w[i], -i});
-  for (int left = blocks - n; left > 0; --left) {
+  for (int i = 0; i < n; ++i) q.push({w[i] / nb[i], -i});
+  for (; left > 0; --left) {
     const int i = -q.top().second;
     q.pop();
     nb[i] += 1;
@@ -132,12 +142,52 @@ static ccm_status check_barrier(ccm_batch b, const char* what) {
   return CCM_OK;
 }
 
-// Entries and block map of the scaled Poisson launch (k_sc_batch for FP64, k_mixed_batch for
-// MIXED), copied to the device; returns once the copies have completed.
+// Entries and block map of the scaled Poisson launch (k_fused_batch or k_sc_batch for FP64,
+// k_mixed_batch for MIXED), copied to the device; returns once the copies have completed.
 static ccm_status upload_poisson_tables(ccm_batch b, bool mixed) {
   const std::vector<ccm_case>& cs = b->cases;
   const int n = (int)cs.size();
   std::vector<int> b0, nb;
+  b->fused = false;
+  if (!mixed && n <= fused_batch_blocks()) {
+    // resident tiles, if every case's fit: each case gets the blocks its tiles need to stay
+    // resident, and the rest goes by weight
+    const int most = std::min(b->blocks, fused_batch_blocks());
+    std::vector<FusedBatchEntry> ef(n);
+    std::vector<int> least(n, 1);
+    int total = 0;
+    bool fits = true;
+    for (int i = 0; i < n && fits; ++i) {
+      case_fused_fp64(cs[i], &ef[i].f);
+      ef[i].f.a.bar = Barrier{b->case_bar + (size_t)kCaseBarStride * i, b->bar_err, 2000000000LL};
+      least[i] = (int)(case_cells(cs[i]) / fused_batch_cells()) + 1;
+      while (least[i] <= most && fused_batch_plan(&ef[i].f, least[i]) == 0) least[i]++;
+      total += least[i];
+      fits = total <= most;
+    }
+    if (fits) allocate_blocks(cell_weights(cs, b->split_exp), most, b0, nb, &least);
+    std::vector<int> block_case;
+    size_t smem = 0;
+    for (int i = 0; i < n && fits; ++i) {
+      const size_t need = fused_batch_plan(&ef[i].f, nb[i]);
+      fits = need > 0;
+      smem = std::max(smem, need);
+      ef[i].block0 = (int)block_case.size();
+      if (fits) block_case.insert(block_case.end(), ef[i].f.ntiles, i);
+    }
+    if (fits) {
+      b->fused = true;
+      b->fused_nblocks = (int)block_case.size();
+      b->fused_smem = smem;
+      cudaError_t e = cudaMemcpyAsync(b->block_case, block_case.data(), sizeof(int) * block_case.size(),
+                                      cudaMemcpyHostToDevice, b->st);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->efu, ef.data(), sizeof(FusedBatchEntry) * n, cudaMemcpyHostToDevice, b->st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);  // the host tables must outlive the copies
+      if (e != cudaSuccess) return bfail(CCM_E_CUDA, std::string("batched Poisson tables: ") + cudaGetErrorString(e));
+      return CCM_OK;
+    }
+  }
   allocate_blocks(cell_weights(cs, b->split_exp), b->blocks, b0, nb);
   std::vector<int> block_case(b->blocks);
   for (int i = 0; i < n; ++i)
@@ -173,6 +223,7 @@ static ccm_status upload_poisson_tables(ccm_batch b, bool mixed) {
 static cudaError_t launch_poisson_scaled(ccm_batch b, bool mixed) {
   BatchControl ctl{b->partials, b->running, Barrier{b->bar_count, b->bar_err, 2000000000LL}, b->case_bar,
                    (int)b->cases.size()};
+  if (!mixed && b->fused) return run_fused_batch(b->efu, b->block_case, ctl, b->fused_nblocks, b->fused_smem, b->st);
   return mixed ? run_mixed_batch(b->emx, b->block_case, ctl, b->blocks, b->st)
                : run_scaled_batch(b->esc, b->block_case, ctl, b->blocks, b->st);
 }
@@ -524,7 +575,8 @@ ccm_status ccm_batch_create(int max_cases, void* stream, ccm_batch* out) {
     delete b;
     return bfail(CCM_E_INVALID, "a batch holds at most " + std::to_string(most) + " cases on this GPU");
   }
-  const size_t pieces[15] = {sizeof(BatchEntry<double>) * max_cases, sizeof(BatchEntry<float>) * max_cases,
+  const size_t pieces[16] = {sizeof(FusedBatchEntry) * max_cases,
+                             sizeof(BatchEntry<double>) * max_cases, sizeof(BatchEntry<float>) * max_cases,
                              sizeof(ScaledBatchEntry) * max_cases, sizeof(MixedBatchEntry) * max_cases,
                              sizeof(int) * b->blocks, sizeof(double) * 6 * b->blocks, sizeof(int) * 2 * b->blocks,
                              sizeof(unsigned int) * kBarWords, sizeof(int) * 4, sizeof(StageCase) * max_cases,
@@ -545,6 +597,7 @@ ccm_status ccm_batch_create(int max_cases, void* stream, ccm_batch* out) {
   b->e32 = (BatchEntry<float>*)take(sizeof(BatchEntry<float>) * max_cases);
   b->esc = (ScaledBatchEntry*)take(sizeof(ScaledBatchEntry) * max_cases);
   b->emx = (MixedBatchEntry*)take(sizeof(MixedBatchEntry) * max_cases);
+  b->efu = (FusedBatchEntry*)take(sizeof(FusedBatchEntry) * max_cases);
   b->block_case = (int*)take(sizeof(int) * b->blocks);
   b->partials = (double*)take(sizeof(double) * 6 * b->blocks);
   b->running = (int*)take(sizeof(int) * 2 * b->blocks);

@@ -122,7 +122,17 @@ struct FusedSolve {
 };
 constexpr int kFusedTilesMax = 512;  // tiles of a launch, at most (two per SM)
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells = 512);
+// One case of a batched launch of resident tiles: its first block (one block per tile).
+struct FusedBatchEntry {
+  FusedSolve f;
+  int block0, pad;
+};
+// Tile plan of a case in a batched launch on at most `blocks` blocks, into *f (a, fxacc, R[0] and
+// the mailboxes set): the dynamic shared memory of its blocks, 0 if its tiles cannot stay resident.
+size_t fused_batch_plan(FusedSolve* f, int blocks);
+int fused_batch_blocks();    // blocks of such a launch, at most
+size_t fused_batch_cells();  // no tile of one has more cells
+void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells = 512, int max_tx = 512);
 int fused_blocks();
 size_t fused_resident_smem_min(int TX, int TY);
 bool fused_resident_ok(int TX, int TY, int ntiles);
@@ -385,6 +395,9 @@ cudaError_t project_zero_mean(const Geom& g, const int8_t* act, double* x, doubl
                               cudaStream_t st);
 cudaError_t run_scaled_batch(const ScaledBatchEntry* dev_cases, const int* dev_block_case, BatchControl ctl,
                              int blocks, cudaStream_t st);
+// smem: the largest of the cases' fused_batch_plan
+cudaError_t run_fused_batch(const FusedBatchEntry* dev_cases, const int* dev_block_case, BatchControl ctl, int blocks,
+                            size_t smem, cudaStream_t st);
 cudaError_t run_mixed_batch(const MixedBatchEntry* dev_cases, const int* dev_block_case, BatchControl ctl,
                             int blocks, cudaStream_t st);
 template <class T>
@@ -400,6 +413,7 @@ int case_nx(ccm_case c);
 void case_poisson_fp64(ccm_case c, PoissonSolve<double>* a);
 bool case_scaled_ok(ccm_case c);  // nonsingular: the scaled and mixed batched kernels apply
 void case_scaled_fp64(ccm_case c, ScaledSolve* a);
+void case_fused_fp64(ccm_case c, FusedSolve* f);  // the same solve on tiles (plan, partials and bar unset)
 void case_mixed_batch(ccm_case c, MixedSolve* a);
 void case_helm_solve(ccm_case c, HelmCSolve* a);
 void case_stage_case(ccm_case c, StageCase* e, int ahead);

@@ -57,6 +57,7 @@
 #include <algorithm>
 
 #include "pcg_common.cuh"
+#include "batch_common.cuh"
 #include "pcg_scalar.cuh"
 
 namespace ccm {
@@ -731,14 +732,26 @@ __global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f2(const __grid_c
   fused_body<true, NT>(f, blockIdx.x, sh);
 }
 
+// Many cases in one cooperative launch: block b serves a tile of case block_case[b], whose tiles
+// pass barriers and words of their own, so every case iterates at its own pace and its blocks leave
+// the launch when it has converged.
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT + 32, MINB) k_fused_batch(const FusedBatchEntry* __restrict__ cases,
+                                                              const int* __restrict__ block_case) {
+  __shared__ FusedShared<NT> sh;
+  __shared__ __align__(16) unsigned char s_entry[sizeof(FusedBatchEntry)];
+  const FusedBatchEntry& E = stage_entry(cases, block_case, s_entry);
+  fused_body<true, NT>(E.f, (int)blockIdx.x - E.block0, sh);
+}
+
 }  // namespace
 
-// Tile shape for at most `blocks` blocks: TX a power of two in 32..512, as many tile rows as
+// Tile shape for at most `blocks` blocks: TX a power of two in 32..max_tx, as many tile rows as
 // the blocks allow while a tile keeps about min_cells cells; the shape with the smallest
 // largest tile wins (then the shortest ring).  One block per tile.
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells) {
+void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells, int max_tx) {
   long long best = -1, best_ring = 0;
-  for (int tx = 32; tx <= 512; tx *= 2) {
+  for (int tx = 32; tx <= max_tx; tx *= 2) {
     const int bxn = (nx + tx - 1) / tx;
     if (bxn > blocks) continue;
     const int wx = std::min(tx, nx);
@@ -863,6 +876,56 @@ size_t fused_mail_slots_max(int nx, int ny) {
 
 // Cells of a built-in resident tile, at least about.
 constexpr int kResidentCells = 128;
+
+// Batched launch: two blocks of 256 computing threads per SM.  Blocks of different cases share an
+// SM, and one's vectors fill the FP64 pipe while the other waits for its reduction.
+constexpr int kBatchNT = 256, kBatchPerSM = 2;
+
+int fused_batch_blocks() { return kBatchPerSM * sm_count(); }
+
+namespace {
+// dynamic shared memory that each of the blocks of an SM can have
+size_t batch_room() {
+  int dev = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  const size_t fixed = sizeof(FusedShared<kBatchNT>) + sizeof(FusedBatchEntry) + 1024 + 256;  // static and reserved
+  return (size_t)per_sm / kBatchPerSM > fixed ? (size_t)per_sm / kBatchPerSM - fixed : 0;
+}
+}  // namespace
+
+size_t fused_batch_cells() { return batch_room() / (5 * sizeof(double) + sizeof(int)) + 1; }
+
+size_t fused_batch_plan(FusedSolve* f, int blocks) {
+  f->ntiles = 0;
+  fused_tiles(f->a.g.nx, f->a.g.ny, blocks, &f->TX, &f->TY, &f->nbx, &f->ntiles, kResidentCells, kBatchNT);
+  if (f->ntiles < 1 || f->ntiles > blocks || f->TX * f->TY > 32 * kBatchNT) return 0;
+  if (f->mail_slots < fused_mail_slots(f->a.g.nx, f->TX, f->TY, f->ntiles)) return 0;
+  f->resident = 1;
+  f->wx = std::min(f->TX, f->a.g.nx);
+  f->list_cap = f->TX * f->TY;
+  const size_t room = batch_room();
+  for (int k = 7; k >= 0; --k) {
+    const size_t smem = resident_smem(f->TX, f->TY, kBatchNT, (k & 4) != 0, (k & 2) != 0, (k & 1) != 0);
+    if (smem > room) continue;
+    f->dcache = (k & 4) != 0;
+    f->defer = (k & 2) != 0;
+    f->lcache = (k & 1) != 0;
+    return smem;
+  }
+  return 0;
+}
+
+cudaError_t run_fused_batch(const FusedBatchEntry* dev_cases, const int* dev_block_case, BatchControl ctl, int blocks,
+                            size_t smem, cudaStream_t st) {
+  if (!ctl.case_bar || ctl.ncases < 1) return cudaErrorInvalidValue;
+  const void* kern = (const void*)k_fused_batch<kBatchNT, kBatchPerSM>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaMemsetAsync(ctl.case_bar, 0, sizeof(unsigned int) * kCaseBarStride * (size_t)ctl.ncases, st);
+  void* params[] = {(void*)&dev_cases, (void*)&dev_block_case};
+  return cudaLaunchCooperativeKernel(kern, blocks, kBatchNT + 32, params, smem, st);
+}
 
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   const int blocks = fused_blocks(), sms = sm_count();

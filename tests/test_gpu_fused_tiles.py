@@ -50,3 +50,30 @@ def test_resident_tiles_at_the_edges_of_the_launch_rules(orc, nx, ny, tx, ty, st
         g.close()
     assert abs(its[0] - its[1]) <= 1
     assert np.linalg.norm(phi[0] - phi[1]) <= 1e-9 * np.linalg.norm(phi[1])
+
+
+@pytest.mark.parametrize("sizes", [[(40, 24), (300, 150), (33, 61)],                 # resident tiles
+                                   [(64, 32)] * 40 + [(512, 256)],                   # ... of many cases and a large one
+                                   [(1024, 512), (1024, 300), (128, 64)]])           # too many cells: vectors in global memory
+def test_fp64_batch_on_both_sides_of_the_resident_limit(sizes):
+    """A batched FP64 step gives each case's own step (solver tolerance apart)."""
+    def make(nx, ny):
+        c = I.small_cylinder(nx=nx, ny=ny, box=(-2.0, 6.0, -2.0, 2.0), r=0.5, cx=0.1, cy=-0.05)
+        c.tol_p, c.tol_h, c.autotune = 1e-11, 1e-12, 0
+        return ccm.Case(c)
+
+    alone, mixed = [make(*s) for s in sizes], [make(*s) for s in sizes]
+    b = ccm.Batch(len(sizes))
+    for c in mixed:
+        b.add(c)
+    for _ in range(2):
+        assert all(s["converged"] for s in b.step(1))
+    pairs = list(zip(alone, mixed))
+    for c, m in pairs[:1] + pairs[1:][-4:]:
+        c.step(2)
+        for f in (ccm.CCM_F_U, ccm.CCM_F_V, ccm.CCM_F_P):
+            a, got = c.get_field(f), m.get_field(f)
+            assert np.linalg.norm(a - got) <= 1e-7 * np.linalg.norm(a), (m.spec.nx, f)
+    b.close()
+    for c in alone + mixed:
+        c.close()
