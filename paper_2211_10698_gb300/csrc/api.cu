@@ -74,6 +74,7 @@ struct ccm_case_s {
   unsigned long long* fxacc;  // words of the fixed-point reduce-barrier (pcg_fixed.cuh)
   ulonglong2* mail;           // mailboxes of the resident tiles (pcg_fused.cu), mail_slots of them
   size_t mail_slots = 0;
+  ulonglong2* bpart;          // partial sums of the resident band tiles (pcg_band.cu)
   int* bar_err;
   DevStats* ds;
   bool geometry = false;
@@ -186,6 +187,7 @@ void carve(ccm_case c, Carver& cv) {
   c->fxacc = cv.take<unsigned long long>(kFxAccWords);
   c->mail_slots = fused_mail_slots_max(c->g.nx, c->g.ny);
   c->mail = cv.take<ulonglong2>(c->mail_slots);
+  c->bpart = cv.take<ulonglong2>(2 * kBandTilesMax);
   c->bar_err = cv.take<int>(4);
   c->ds = cv.take<DevStats>(1);
   c->hs_u = cv.take<double>(N);
@@ -424,6 +426,16 @@ void case_mixed1_solve(ccm_case c, const MixedSolve& a, const TilePlan& tp, Mixe
   f->resident = tp.resident;
 }
 
+// The resident form (pcg_band.cu); pz and pp0 are FP64 work arrays that mixed solves do not use.
+void case_band_solve(ccm_case c, const MixedSolve& a, BandSolve* f) {
+  *f = BandSolve{};
+  f->m = a;
+  f->WT[0] = (unsigned long long*)c->pz;
+  f->WT[1] = (unsigned long long*)c->pp0;
+  f->E = c->fx;
+  f->part = c->bpart;
+}
+
 ccm_status solve_poisson_mixed(ccm_case c, double* x, double* b) {
   // periodic sides: the host-driven refinement on the general kernel, which writes the images
   if (!c->zero_mean && !c->g.px && !c->g.py) {
@@ -431,7 +443,11 @@ ccm_status solve_poisson_mixed(ccm_case c, double* x, double* b) {
     // Chebyshev preconditioner), with one grid barrier per iteration when the tuner chose it
     MixedSolve a{};
     case_mixed_solve(c, x, b, &a);
-    if (c->tune.mixed1.TX > 0) {
+    BandSolve bs{};
+    case_band_solve(c, a, &bs);
+    if (c->tune.mixed1.TX == 0 && c->tune.mixed_blocks == 0 && band_fits(&bs)) {
+      CUDA_TRY(run_poisson_band(bs, c->st));
+    } else if (c->tune.mixed1.TX > 0) {
       Mixed1Solve f{};
       case_mixed1_solve(c, a, c->tune.mixed1, &f);
       CUDA_TRY(run_poisson_mixed1(f, c->st));
@@ -521,17 +537,30 @@ ccm_status autotune_poisson(ccm_case c) {
   std::vector<float> ms;
   cudaError_t e = cudaSuccess;
   if (mixed) {
-    // block counts of the mixed solve, then tile plans of its one-barrier form
-    const std::vector<int> cand = mixed_block_candidates(most);
-    const std::vector<TilePlan> cand1 = mixed1_plan_candidates(g.nx, g.ny, deg);
-    const int nm = (int)cand.size();
+    // Block counts of the mixed solve, then the resident band tiles where they fit, else the tile
+    // plans of the one-barrier form: from 16x12 to 2048x1024 the band tiles took 0.5 to 0.8 of the
+    // time of its best plan.  The band's start-up is longer than a few iterations, so the candidates
+    // run more of them.
     MixedSolve a{};
     case_mixed_solve(c, x, b, &a);
     a.d.tol = 0.0;
     a.d.max_iter = kTuneIters;
-    e = time_launches(nm + (int)cand1.size(), [&](int k) -> cudaError_t {
+    BandSolve bs{};
+    case_band_solve(c, a, &bs);
+    const bool band = band_fits(&bs);
+    const std::vector<int> cand = mixed_block_candidates(most);
+    const std::vector<TilePlan> cand1 = band ? std::vector<TilePlan>{} : mixed1_plan_candidates(g.nx, g.ny, deg);
+    const int nm = (int)cand.size(), nm1 = nm + (int)cand1.size();
+    if (band) {
+      a.d.max_iter = bs.m.d.max_iter = 4 * kTuneIters;
+      // untimed: a kernel's first launch loads it
+      CUDA_TRY(cudaMemsetAsync(x, 0, bytes, st));
+      CUDA_TRY(run_poisson_band(bs, st));
+    }
+    e = time_launches(nm1 + (band ? 1 : 0), [&](int k) -> cudaError_t {
       cudaError_t me = cudaMemsetAsync(x, 0, bytes, st);
       if (me != cudaSuccess) return me;
+      if (k >= nm1) return run_poisson_band(bs, st);
       if (k >= nm) {
         Mixed1Solve f{};
         case_mixed1_solve(c, a, cand1[k - nm], &f);
@@ -540,7 +569,8 @@ ccm_status autotune_poisson(ccm_case c) {
       a.blocks = cand[k];
       return run_poisson_mixed(a, st);
     }, st, &best, &ms);
-    if (best >= nm) r.mixed1 = cand1[best - nm];
+    if (best >= nm1) r.band = bs.ntiles;
+    else if (best >= nm) r.mixed1 = cand1[best - nm];
     else if (best >= 0) r.mixed_blocks = cand[best];
   } else {
     const std::vector<TilePlan> cand = fused_plan_candidates(g.nx, g.ny, most);
@@ -917,7 +947,7 @@ ccm_status ccm_launch_plan(ccm_case c, int plan[7]) {
   plan[1] = tp.TY;
   plan[2] = tp.nbx;
   plan[3] = tp.ntiles;
-  plan[4] = c->tune.mixed_blocks;
+  plan[4] = c->tune.band > 0 ? c->tune.band : c->tune.mixed_blocks;
   plan[5] = c->tune.cluster;
   plan[6] = tp.resident;
   return CCM_OK;
@@ -961,7 +991,15 @@ ccm_status ccm_set_launch_plan(ccm_case c, const int plan[7]) {
     return fail(CCM_E_INVALID, "resident tiles need a tile plan");
   }
   if (plan[4] < 0 || plan[4] > mixed_blocks()) return fail(CCM_E_INVALID, "mixed blocks out of range");
-  r.mixed_blocks = plan[4];
+  // as many blocks as the resident band has tiles: that solve, as ccm_launch_plan reports it
+  if (mixed && plan[4] > 0 && !c->zero_mean && !c->g.px && !c->g.py) {
+    MixedSolve a{};
+    case_mixed_solve(c, nullptr, nullptr, &a);
+    BandSolve bs{};
+    case_band_solve(c, a, &bs);
+    if (band_fits(&bs) && bs.ntiles == plan[4]) r.band = plan[4];
+  }
+  if (r.band == 0) r.mixed_blocks = plan[4];
   if (plan[5] != 0) {
     bool ok = false;
     for (int C : cluster_candidates(g.nx, g.ny)) ok = ok || C == plan[5];

@@ -159,6 +159,7 @@ struct TuneResult {
   int mixed_blocks;  // mixed one-launch solve (0: not tuned)
   int cluster;       // FP64 solve inside one cluster of this many CTAs (0: not chosen)
   TilePlan mixed1;   // mixed solve with one barrier per iteration (TX = 0: not chosen)
+  int band;          // mixed solve on resident band tiles: their number (0: not chosen)
 };
 std::vector<TilePlan> fused_plan_candidates(int nx, int ny, int blocks);
 std::vector<int> mixed_block_candidates(int blocks);
@@ -217,6 +218,23 @@ size_t mixed1_smem(int TX, int TY, int cheb, int resident);
 bool mixed1_plan_fits(int TX, int TY, int ntiles, int cheb, int resident);
 // Tile plans of the one-barrier mixed solve that fit the GPU at once, resident ones first.
 std::vector<TilePlan> mixed1_plan_candidates(int nx, int ny, int cheb);
+
+// The same mixed solve on resident tiles with their band (pcg_band.cu): no FP32 vector in global
+// memory but the frames that neighbours exchange.  m.d.x, m.d.b, m.d.r (FP64 residual),
+// m.d.partials and the scalars of m are used; m's FP32 vectors are not.
+struct BandSolve {
+  MixedSolve m;
+  unsigned long long* WT[2];  // K~ u of the frames, value and tag, by parity of the apply (a word per cell)
+  float* E;                   // correction
+  ulonglong2* part;           // 2 x kBandTilesMax slots of tagged partial sums
+  int W, TY, nbx, ntiles;     // tile plan (band_plan)
+  int shape;                  // warps and region rows per warp (pcg_band.cu)
+  int ncut;                   // shared-memory slots for the coefficients of cut quads
+};
+constexpr int kBandTilesMax = 512;
+// The tile plan of a single solve into *f (f->m set); false if the tiles cannot stay resident.
+bool band_fits(BandSolve* f);
+cudaError_t run_poisson_band(BandSolve f, cudaStream_t st);
 
 // One case of a batched solve and its contiguous range of blocks (pcg_batch.cu).
 struct ScaledBatchEntry {
