@@ -168,6 +168,7 @@ void carve(ccm_case c, Carver& cv) {
   for (double** q : {&o.sdk, &o.isdk, &o.cus, &o.cvs}) *q = cv.take<double>(N);
   for (float** q : {&o.isdk32, &o.cus32, &o.cvs32}) *q = cv.take<float>(N);
   o.kinds = cv.take<int8_t>(N);
+  o.kindq = cv.take<int8_t>(N);
   double** st[] = {&c->u, &c->v, &c->p, &c->phi, &c->cnu[0], &c->cnu[1], &c->cnv[0], &c->cnv[1],
                    &c->ustar, &c->vstar, &c->div, &c->rhs_u, &c->rhs_v, &c->rhs_p,
                    &c->pr, &c->pz, &c->pp0, &c->pp1, &c->pq, &c->pz2, &c->pw1,
@@ -404,7 +405,7 @@ void case_mixed_solve(ccm_case c, double* x, const double* b, MixedSolve* a) {
   a->d.partials = c->partials;
   a->d.bar = case_barrier(c);
   a->d.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, &c->ds->total_p, &c->ds->nconv};
-  a->cus32 = c->co.cus32; a->cvs32 = c->co.cvs32;
+  a->cus32 = c->co.cus32; a->cvs32 = c->co.cvs32; a->kindq = c->co.kindq;
   a->r = c->fr; a->w = c->fq; a->p = c->fp0; a->s = c->fp1; a->e = c->fx;
   a->cheb = c->cfg.precond == CCM_CHEBYSHEV ? c->cfg.cheb_degree : 1;
   a->zA = c->fz2; a->zB = c->fw1; a->dch = c->fb;

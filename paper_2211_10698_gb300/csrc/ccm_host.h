@@ -31,6 +31,9 @@ struct CoefPtrs {
   double *sdk, *isdk, *cus, *cvs;
   float *isdk32, *cus32, *cvs32;
   int8_t* kinds;
+  // kinds of the FP32 rows: 3 for a cut row whose coefficients are the constant stencil's in FP32
+  // (one that the rounding of the abscissas alone marks as cut), which then need not be read
+  int8_t* kindq;
 };
 
 // Where a solver kernel reports: iterations, final squared residual and right-hand side
@@ -177,6 +180,7 @@ cudaError_t time_launches(int n, const std::function<cudaError_t(int)>& launch, 
 struct MixedSolve {
   ScaledSolve d;
   const float *cus32, *cvs32;
+  const int8_t* kindq;
   float *r, *w, *p, *s, *e;   // FP32 residual, K~ u, direction, K~ p, correction
   int cheb;                   // 1: Jacobi (u = r); k > 1: k-step Chebyshev preconditioner
   float *zA, *zB, *dch;       // Chebyshev iterates and direction (cheb > 1)

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   // the FP32 phases work on aligned quads of the case's arrays (see QuadOpsF32)
   const Quads Q(g);
   const int u0 = (int)((long long)Q.nquad * lb / nbc), u1 = (int)((long long)Q.nquad * (lb + 1) / nbc);
-  const QuadOpsF32 ops{d.kinds, A.cus32, A.cvs32, (float)d.ax, (float)d.ay, g.pitch};
+  const QuadOpsF32 ops{A.kindq, A.cus32, A.cvs32, (float)d.ax, (float)d.ay, g.pitch};
   const double* __restrict__ r64 = d.r;
   float* __restrict__ r = A.r;
   float* __restrict__ w = A.w;

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_pcg_poisson_mixed(MixedSolve
   const Quads Q(g);
   const int u0 = (int)((long long)Q.nquad * blockIdx.x / gridDim.x);
   const int u1 = (int)((long long)Q.nquad * (blockIdx.x + 1) / gridDim.x);
-  const QuadOpsF32 ops{d.kinds, a.cus32, a.cvs32, (float)d.ax, (float)d.ay, P};
+  const QuadOpsF32 ops{a.kindq, a.cus32, a.cvs32, (float)d.ax, (float)d.ay, P};
   const int first = ch.t0 + threadIdx.x, stride = blockDim.x;
   const double* __restrict__ isd = d.isd;
   double* __restrict__ x = d.x;

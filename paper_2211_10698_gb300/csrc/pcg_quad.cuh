@@ -42,7 +42,7 @@ struct Quads {
 };
 
 struct QuadOpsF32 {
-  const int8_t* kinds;
+  const int8_t* kinds;  // kindq: 0 identity, 1 constant stencil, 2 own coefficients, 3 own, equal to the constants
   const float* cus;
   const float* cvs;
   float ax, ay;
@@ -50,10 +50,12 @@ struct QuadOpsF32 {
 
   // Scaled face coefficients of the quad (W faces, E face of the last cell, S faces, N faces).
   // Only rows of kind 2 (cut) use them, so a quad without one loads none: on the uniform
-  // part of the grid the stencil reads its vector and the kinds only.
+  // part of the grid the stencil reads its vector and the kinds only; rows of kind 3 have the
+  // constants for coefficients and take them in the cut rows' formula, the same bits as read.
   __device__ __forceinline__ void coefs(int k0, const char4& km, float4& cw, float& ce4, float4& cs, float4& cn) const {
-    cw = cs = cn = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    ce4 = 0.0f;
+    cw = make_float4(ax, ax, ax, ax);
+    cs = cn = make_float4(ay, ay, ay, ay);
+    ce4 = ax;
     if (km.x == 2 || km.y == 2 || km.z == 2 || km.w == 2) {
       cw = ld4(cus, k0);
       cs = ld4(cvs, k0);
@@ -76,7 +78,7 @@ struct QuadOpsF32 {
       const float ce = m == 3 ? ce4 : at(cw, m + 1);
       const float wu = c - ax * (l + rr) - ay * (sv + nv);
       const float wg = c - at(cw, m) * l - ce * rr - at(cs, m) * sv - at(cn, m) * nv;
-      put(out, m, kk == 1 ? wu : (kk == 2 ? wg : c));
+      put(out, m, kk == 1 ? wu : (kk >= 2 ? wg : c));
     }
     return out;
   }
