@@ -1101,10 +1101,9 @@ ccm_status ccm_set_geometry(ccm_case c, const ccm_geometry* geo) {
   launch_fill_bc(g, c->bc, c->t0, c->t1, 1.0, st);
   launch_visc(c->cv, g, c->bc, c->t0, c->t1, c->co.liftu, c->co.liftv, st);
   // Jacobi diagonal of the Helmholtz operator by colour probing
-  launch_helmholtz_diag(c->cv, g, c->bc, c->ph, c->t0, c->t1, c->t2, c->t3, c->t4, c->t5, c->co.invdhu, c->co.invdhv,
-                        st);
+  launch_helmholtz_diag(c->cv, g, c->bc, c->ph, c->t4, c->t5, c->co.invdhu, c->co.invdhv, st);
   // its nine coefficients per unknown face, by colour probing
-  launch_helmholtz_coefs(c->cv, g, c->bc, c->ph, c->t0, c->t1, c->t2, c->t3, c->hc, c->hc_bad, st);
+  launch_helmholtz_coefs(c->cv, g, c->bc, c->ph, c->hc, c->hc_bad, st);
   // state
   const size_t bytes = g.count() * sizeof(double);
   for (double* a : {c->p, c->phi, c->cnu[0], c->cnu[1], c->cnv[0], c->cnv[1], c->ustar, c->vstar, c->div})
@@ -1290,7 +1289,7 @@ ccm_status ccm_apply_op(ccm_case c, int op, const double* in0, const double* in1
       break;
     case CCM_OP_HELMHOLTZ_DIAG:
       if (!need(out0) || !need(out1)) return fail(CCM_E_INVALID, "needs out0, out1");
-      launch_helmholtz_diag(c->cv, g, c->bc, c->ph, c->t0, c->t1, c->t2, c->t3, c->t4, c->t5, nullptr, nullptr, st);
+      launch_helmholtz_diag(c->cv, g, c->bc, c->ph, c->t4, c->t5, nullptr, nullptr, st);
       if ((s = download(c, out0, c->t4)) || (s = download(c, out1, c->t5))) return s;
       break;
     default:

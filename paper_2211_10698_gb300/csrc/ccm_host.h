@@ -277,8 +277,8 @@ struct BatchControl {
 struct HelmCoefPtrs {
   double* a[18];
 };
-void launch_helmholtz_coefs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* eu, double* ev,
-                            double* ou, double* ov, const HelmCoefPtrs& h, int* bad, cudaStream_t st);
+void launch_helmholtz_coefs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, const HelmCoefPtrs& h, int* bad,
+                            cudaStream_t st);
 
 // Helmholtz PCG on the coefficient form (pcg_helm.cu): single-reduction Jacobi CG over the
 // unknown u and v faces.
@@ -374,8 +374,8 @@ void launch_visc(const Coefs& c, const Geom& g, const Bc& bc, const double* u, c
 void launch_helmholtz(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, const double* u, const double* v,
                       double* ou, double* ov, cudaStream_t st);
 void launch_poisson(const Coefs& c, const Geom& g, const double* x, double* out, double* tmp, cudaStream_t st);
-void launch_helmholtz_diag(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* eu, double* ev,
-                           double* ou, double* ov, double* du, double* dv, double* iu, double* iv, cudaStream_t st);
+void launch_helmholtz_diag(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* du, double* dv,
+                           double* iu, double* iv, cudaStream_t st);
 void launch_predictor_rhs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, const double* u, const double* v,
                           const double* p, const double* cpu, const double* cpv, double* cnu, double* cnv, double* ru,
                           double* rv, int first, cudaStream_t st);

@@ -300,9 +300,21 @@ __device__ __forceinline__ void grid_sum(const double* partials, int nblocks, do
 // Homogeneous view of a velocity-like vector: value on unknowns, zero on Dirichlet and
 // inactive faces, and on ghost positions the zero-gradient copy or the reflection of the
 // adjacent position according to the side's boundary type.
-struct HomView {
+struct ArraySource {
   const double* u;
   const double* v;
+  __device__ __forceinline__ double u_of(int, int, size_t k) const { return u[k]; }
+  __device__ __forceinline__ double v_of(int, int, size_t k) const { return v[k]; }
+};
+// Ones on the positions of component comp whose indices are congruent to (a, b) mod 3.
+struct ProbeSource {
+  int comp, a, b;
+  __device__ __forceinline__ bool on(int i, int j) const { return (i + 3) % 3 == a && (j + 3) % 3 == b; }
+  __device__ __forceinline__ double u_of(int i, int j, size_t) const { return comp == 0 && on(i, j) ? 1.0 : 0.0; }
+  __device__ __forceinline__ double v_of(int i, int j, size_t) const { return comp == 1 && on(i, j) ? 1.0 : 0.0; }
+};
+template <class Source>
+struct HomViewOf : Source {
   const int8_t* ru;
   const int8_t* rv;
   Geom g;
@@ -316,7 +328,7 @@ struct HomView {
     else if (j < 0) { j = 0; if (bc.type[CCM_SIDE_S] == CCM_BC_DIRICHLET) s = -1.0; }
     else if (j >= g.ny) { j = g.ny - 1; if (bc.type[CCM_SIDE_N] == CCM_BC_DIRICHLET) s = -1.0; }
     size_t k = g.idx(i, j);
-    return ru[k] == R_UNKNOWN ? s * u[k] : 0.0;
+    return ru[k] == R_UNKNOWN ? s * this->u_of(i, j, k) : 0.0;
   }
   __device__ __forceinline__ double at_v(int i, int j) const {
     double s = 1.0;
@@ -327,9 +339,11 @@ struct HomView {
     else if (i < 0) { i = 0; if (bc.type[CCM_SIDE_W] == CCM_BC_DIRICHLET) s = -1.0; }
     else if (i >= g.nx) { i = g.nx - 1; if (bc.type[CCM_SIDE_E] == CCM_BC_DIRICHLET) s = -1.0; }
     size_t k = g.idx(i, j);
-    return rv[k] == R_UNKNOWN ? s * v[k] : 0.0;
+    return rv[k] == R_UNKNOWN ? s * this->v_of(i, j, k) : 0.0;
   }
 };
+
+using HomView = HomViewOf<ArraySource>;
 
 // Full view: the arrays already hold Dirichlet faces and ghosts (filled by fill_bc).
 struct FullView {

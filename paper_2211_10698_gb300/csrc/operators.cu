@@ -209,28 +209,37 @@ __global__ void k_copy_interior_cells(Geom g, const double* in, double* out) {
   out[k] = dom ? in[k] : 0.0;
 }
 
-// Probe vectors for diag(H): ones on the unknown and inactive positions of one component
-// whose indices are congruent to (a, b) mod 3 (H couples positions at distance <= 1).
-__global__ void k_probe_set(Coefs c, Geom g, int comp, int a, int b, double* eu, double* ev) {
-  PAD_IJ(g)
-  const bool col = ((i + 3) % 3 == a) && ((j + 3) % 3 == b);
-  eu[k] = (comp == 0 && col && c.role_u[k] >= R_INACTIVE) ? 1.0 : 0.0;
-  ev[k] = (comp == 1 && col && c.role_v[k] >= R_INACTIVE) ? 1.0 : 0.0;
+// H of the probe vectors (ones on the unknown and inactive positions of one component whose indices
+// are congruent to (a, b) mod 3; H couples positions at distance <= 1) is evaluated where it is read,
+// from a view that knows the probe: neither the 18 vectors nor their images pass through memory, and
+// the diagonal costs one row evaluation per position, not 18.  Diagonal and coefficients took 108
+// launches (128x64: 0.7 of a set-up's 1.3 ms; 512x256: 0.8 of 2.2 ms) and take three.
+__device__ __forceinline__ double helm_row_u(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph,
+                                             const HomViewOf<ProbeSource>& w, int i, int j, size_t k) {
+  return c.massu[k] * w.u_of(i, j, k) - ph.mu * visc_u(c, g, bc, w, i, j);
 }
-__global__ void k_probe_get(Coefs c, Geom g, int comp, int a, int b, const double* ou, const double* ov, double* du,
-                            double* dv) {
+__device__ __forceinline__ double helm_row_v(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph,
+                                             const HomViewOf<ProbeSource>& w, int i, int j, size_t k) {
+  return c.massv[k] * w.v_of(i, j, k) - ph.mu * visc_v(c, g, bc, w, i, j);
+}
+// diag(H): every position's response to the probe of its own colour (1 on inactive positions, 0
+// elsewhere)
+__global__ void k_helm_diag(Coefs c, Geom g, Bc bc, Phys ph, double* du, double* dv) {
   PAD_IJ(g)
-  const bool col = ((i + 3) % 3 == a) && ((j + 3) % 3 == b);
-  if (comp == 0 && col && c.role_u[k] >= R_INACTIVE) du[k] = ou[k];
-  if (comp == 1 && col && c.role_v[k] >= R_INACTIVE) dv[k] = ov[k];
+  const int a = (i + 3) % 3, b = (j + 3) % 3;
+  const int8_t ru = c.role_u[k], rv = c.role_v[k];
+  const HomViewOf<ProbeSource> wu{{0, a, b}, c.role_u, c.role_v, g, bc}, wv{{1, a, b}, c.role_u, c.role_v, g, bc};
+  du[k] = ru == R_UNKNOWN ? helm_row_u(c, g, bc, ph, wu, i, j, k) : (ru == R_INACTIVE ? 1.0 : 0.0);
+  dv[k] = rv == R_UNKNOWN ? helm_row_v(c, g, bc, ph, wv, i, j, k) : (rv == R_INACTIVE ? 1.0 : 0.0);
 }
 // Coefficient extraction: after applying the operator to the unit vector of colour (a, b) of
 // component comp, row (i, j) sees exactly one unit inside its 3x3 neighbourhood, at the offset
 // (di, dj) with i + di = a, j + dj = b (mod 3); its response is the coefficient of that
 // neighbour.  A response at an offset outside the row's pattern is flagged in *bad.
-__global__ void k_probe_coef(Coefs c, Geom g, int comp, int a, int b, const double* ou, const double* ov,
-                             HelmCoefPtrs h, int* bad) {
+__global__ void k_helm_coef(Coefs c, Geom g, Bc bc, Phys ph, HelmCoefPtrs h, int* bad) {
   PAD_IJ(g)
+  const int comp = blockIdx.z / 9, a = blockIdx.z / 3 % 3, b = blockIdx.z % 3;
+  const HomViewOf<ProbeSource> w{{comp, a, b}, c.role_u, c.role_v, g, bc};
   auto off = [](int want, int at) {
     const int d = ((want - at) % 3 + 3) % 3;
     return d == 2 ? -1 : d;
@@ -244,8 +253,9 @@ __global__ void k_probe_coef(Coefs c, Geom g, int comp, int a, int b, const doub
     else
       slot = (di == -1 && dj == 0) ? 5 : (di == 0 && dj == 0) ? 6 : (di == -1 && dj == 1) ? 7
            : (di == 0 && dj == 1) ? 8 : -1;
-    if (slot >= 0) h.a[slot][k] = ou[k];
-    else if (ou[k] != 0.0) atomicOr(bad, 1);
+    const double o = helm_row_u(c, g, bc, ph, w, i, j, k);
+    if (slot >= 0) h.a[slot][k] = o;
+    else if (o != 0.0) atomicOr(bad, 1);
   }
   if (c.role_v[k] == R_UNKNOWN) {
     int slot = -1;
@@ -255,8 +265,9 @@ __global__ void k_probe_coef(Coefs c, Geom g, int comp, int a, int b, const doub
     else
       slot = (di == 0 && dj == -1) ? 14 : (di == 1 && dj == -1) ? 15 : (di == 0 && dj == 0) ? 16
            : (di == 1 && dj == 0) ? 17 : -1;
-    if (slot >= 0) h.a[slot][k] = ov[k];
-    else if (ov[k] != 0.0) atomicOr(bad, 1);
+    const double o = helm_row_v(c, g, bc, ph, w, i, j, k);
+    if (slot >= 0) h.a[slot][k] = o;
+    else if (o != 0.0) atomicOr(bad, 1);
   }
 }
 __global__ void k_invert_diag(Geom g, const double* du, const double* dv, double* iu, double* iv) {
@@ -647,30 +658,18 @@ void launch_poisson(const Coefs& c, const Geom& g, const double* x, double* out,
   if (g.px || g.py) k_wrap_cells<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, tmp);
   k_poisson<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, tmp, out);
 }
-void launch_helmholtz_diag(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* eu, double* ev,
-                           double* ou, double* ov, double* du, double* dv, double* iu, double* iv, cudaStream_t st) {
-  cudaMemsetAsync(du, 0, g.count() * sizeof(double), st);
-  cudaMemsetAsync(dv, 0, g.count() * sizeof(double), st);
-  for (int comp = 0; comp < 2; ++comp)
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        k_probe_set<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, comp, a, b, eu, ev);
-        launch_helmholtz(c, g, bc, ph, eu, ev, ou, ov, st);
-        k_probe_get<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, comp, a, b, ou, ov, du, dv);
-      }
+void launch_helmholtz_diag(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* du, double* dv,
+                           double* iu, double* iv, cudaStream_t st) {
+  k_helm_diag<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, bc, ph, du, dv);
   if (iu) k_invert_diag<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, du, dv, iu, iv);
 }
-void launch_helmholtz_coefs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, double* eu, double* ev,
-                            double* ou, double* ov, const HelmCoefPtrs& h, int* bad, cudaStream_t st) {
+void launch_helmholtz_coefs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, const HelmCoefPtrs& h, int* bad,
+                            cudaStream_t st) {
   for (int q = 0; q < 18; ++q) cudaMemsetAsync(h.a[q], 0, g.count() * sizeof(double), st);
   cudaMemsetAsync(bad, 0, sizeof(int), st);
-  for (int comp = 0; comp < 2; ++comp)
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        k_probe_set<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, comp, a, b, eu, ev);
-        launch_helmholtz(c, g, bc, ph, eu, ev, ou, ov, st);
-        k_probe_coef<<<pad_grid(g, kBlk), kBlk, 0, st>>>(c, g, comp, a, b, ou, ov, h, bad);
-      }
+  dim3 grd = pad_grid(g, kBlk);
+  grd.z = 18;  // one probe each
+  k_helm_coef<<<grd, kBlk, 0, st>>>(c, g, bc, ph, h, bad);
 }
 void launch_predictor_rhs(const Coefs& c, const Geom& g, const Bc& bc, const Phys& ph, const double* u, const double* v,
                           const double* p, const double* cpu, const double* cpv, double* cnu, double* cnv, double* ru,

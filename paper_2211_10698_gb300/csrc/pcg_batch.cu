@@ -8,7 +8,8 @@
 // blocks pass; a case on one block needs only the block barrier), so every case iterates at
 // its own pace and its blocks leave the launch when it has converged.
 //
-// FP64 solve: two barriers per CG iteration.
+// FP64 solve, of batches whose tiles do not all stay resident (those that do: pcg_fused.cu): two
+// barriers per CG iteration.
 //
 // Mixed solve: each case steps through slots, one barrier after each, according to where it
 // is.  The barrier after a slot is the case's own (a counter per case that only its blocks

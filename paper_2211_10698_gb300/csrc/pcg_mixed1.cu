@@ -3,6 +3,9 @@
 // Jacobi-scaled correction equation, FP64 residual replacements) in the tile layout of
 // pcg_fused.cu, extended to the Chebyshev preconditioner.
 //
+// It serves grids whose tiles and bands do not fit the GPU at once in pcg_band.cu's layout (large
+// ones, stretched ones), and tile plans that a caller sets.
+//
 // pcg_mixed.cu separates every phase that reads neighbours by a grid barrier: the vector
 // update, each of the k-1 Chebyshev steps and the stencil with its sums, i.e. k+1 barriers per
 // iteration.  Here each block owns a 2-D tile and a band of width k around it:

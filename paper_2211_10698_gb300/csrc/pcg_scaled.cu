@@ -42,10 +42,8 @@ __global__ void k_scaling(Geom g, double uncut, CoefPtrs o) {
   o.sdk[k] = sd;
   o.isdk[k] = isd;
   o.isdk32[k] = (float)isd;
-  auto cus_at = [&](size_t q) { return o.cu[q] * isd_at(q) * isd_at(q - 1); };
-  auto cvs_at = [&](size_t q) { return o.cv[q] * isd_at(q) * isd_at(q - g.pitch); };
-  const double cus = i >= 0 ? cus_at(k) : 0.0;
-  const double cvs = j >= 0 ? cvs_at(k) : 0.0;
+  const double cus = i >= 0 ? o.cu[k] * isd * isd_at(k - 1) : 0.0;
+  const double cvs = j >= 0 ? o.cv[k] * isd * isd_at(k - g.pitch) : 0.0;
   o.cus[k] = cus;
   o.cvs[k] = cvs;
   o.cus32[k] = (float)cus;
@@ -69,7 +67,10 @@ __global__ void k_scaling(Geom g, double uncut, CoefPtrs o) {
   if (ks == 2) {
     const double cx = g.hy / g.hx, cy = g.hx / g.hy, dreg = 2.0 * (cx + cy);
     const float ax = (float)(cx / dreg), ay = (float)(cy / dreg);
-    if ((float)cus == ax && (float)cus_at(k + 1) == ax && (float)cvs == ay && (float)cvs_at(k + g.pitch) == ay) ks = 3;
+    // (the E and N neighbours form their W and S faces like this)
+    if ((float)cus == ax && (float)cvs == ay && (float)(o.cu[k + 1] * isd_at(k + 1) * isd) == ax &&
+        (float)(o.cv[k + g.pitch] * isd_at(k + g.pitch) * isd) == ay)
+      ks = 3;
   }
   o.kindq[k] = ks;
 }

@@ -1,7 +1,8 @@
 // Launch-shape autotuner for the one-launch Poisson solves: the tile plan of the FP64 CG with
 // one barrier per iteration (pcg_fused.cu) or, on small grids, the size of the one cluster
-// that holds the whole FP64 solve (pcg_cluster.cu), and the block count of the
-// mixed-precision solve (pcg_mixed.cu).  Which shape is fastest depends on the grid: a large
+// that holds the whole FP64 solve (pcg_cluster.cu), and for the mixed-precision solve the
+// resident band tiles (pcg_band.cu) or the block count of the kernel with a barrier per phase
+// (pcg_mixed.cu).  Which shape is fastest depends on the grid: a large
 // grid wants every SM busy, a small one loses more to the grid barrier across many blocks
 // than it gains from them.  The caller times each candidate on a short solve of the case's
 // own operator (a fixed number of iterations on a scratch right-hand side) and keeps the
