@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   __shared__ float fsum[8];
   __shared__ double sc_sigma, sc_rr, sc_bb, sc_rr_ref, sc_racc[3];
   __shared__ float sc_alpha, sc_beta, sc_pscale, sc_igamma, sc_ialpha, sc_gref, sc_gfresh;
-  __shared__ int sc_slot, sc_part, sc_j, sc_fresh, sc_it, sc_stop, sc_nrep, sc_rep_it, sc_keep, sc_restart, sc_final,
+  __shared__ int sc_slot, sc_part, sc_fresh, sc_it, sc_stop, sc_nrep, sc_rep_it, sc_keep, sc_restart, sc_final,
       sc_init;
   unsigned int target = 0;
   const int NB = gridDim.x;
@@ -279,6 +279,8 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   // the FP32 phases work on aligned quads of the case's arrays (see QuadOpsF32)
   const Quads Q(g);
   const int u0 = (int)((long long)Q.nquad * lb / nbc), u1 = (int)((long long)Q.nquad * (lb + 1) / nbc);
+  // the thread's first quad (of one or two on most batches), found once
+  const int ufirst = u0 + (int)threadIdx.x, kfirst = ufirst < u1 ? Q.k(ufirst) : 0;
   const QuadOpsF32 ops{A.kindq, A.cus32, A.cvs32, (float)d.ax, (float)d.ay, g.pitch};
   const double* __restrict__ r64 = d.r;
   float* __restrict__ r = A.r;
@@ -300,7 +302,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
     sc_bb = 0.0;
     sc_igamma = 1.0f;
     sc_pscale = 1.0f;
-    sc_j = sc_fresh = sc_it = sc_stop = sc_nrep = sc_keep = sc_restart = sc_final = 0;
+    sc_fresh = sc_it = sc_stop = sc_nrep = sc_keep = sc_restart = sc_final = 0;
     sc_rep_it = -1000;
   }
   __syncthreads();
@@ -308,23 +310,24 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   // Slot t publishes its sums in rows 3 (t & 1) .. 3 (t & 1) + 2 of the partials: the rows a
   // slot reads after its barrier are written again two slots later, after a barrier that every
   // block reaches only once it has read them.
+  // The slot after one without sums is known to every thread; after sums thread 0 decides.
+  int sl = SL_FOLD, step = 1;
   for (unsigned int t = 0; ok; ++t) {
-    const int sl = sc_slot, part = sc_part;
+    const int part = sc_part;
     if (sl == SL_DONE) break;  // every block of the case sees the same slot
     const bool last_part = part == nparts - 1;
     double* prow = ctl.partials + (size_t)(3 * (t & 1)) * NB;
     if (sl == SL_FOLD) {
       if (sc_init) {
         const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
-          const int k0 = Q.k(u);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) {
           st4(p, k0, z);
           st4(s, k0, z);
           st4(e, k0, z);
         }
       } else {
         const double isig = 1.0 / sc_sigma;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) quad_fold(d.x, d.isd, e, Q.k(u), isig, true);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) quad_fold(d.x, d.isd, e, k0, isig, true);
       }
     } else if (sl == SL_RESID) {
       // part `part` of the block's cells: r64 = D^-1/2 (b - K x) and the norms, summed over
@@ -354,38 +357,37 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       if (cheb == 1) {
         // r = sigma r64 (FP32), w = K~ r, sums (r, r), (w, r)
         float v[2] = {0.0f, 0.0f};
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.stencil(r, w, r64, sig, Q.k(u), v);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.stencil(r, w, r64, sig, k0, v);
         block_sum_f32<2>(v, wred, fsum);
         const double dv[3] = {(double)fsum[0], (double)fsum[1], (double)fsum[0]};
         publish(prow, NB, dv, 3);
       } else {
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
-          const int k0 = Q.k(u);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) {
           st4(r, k0, ld4_scaled(r64, k0, sig));
         }
       }
     } else if (sl == SL_CHEB) {
-      const int j = sc_j;
+      const int j = step;
       float c1, c2;
       cheb_step_coef(j, c1, c2);
       float* zout = (j & 1) ? A.zB : A.zA;
       if (j == 1) {
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.cheb_first(r, A.dch, zout, Q.k(u), ith, c1, c2);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.cheb_first(r, A.dch, zout, k0, ith, c1, c2);
       } else {
         const float* zin = (j & 1) ? A.zA : A.zB;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.cheb_step(zin, r, A.dch, zout, Q.k(u), c1, c2);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.cheb_step(zin, r, A.dch, zout, k0, c1, c2);
       }
     } else if (sl == SL_APPLY) {
       float v[3] = {0.0f, 0.0f, 0.0f};
       if (cheb == 1) {
         float v2[2] = {0.0f, 0.0f};
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.stencil(r, w, nullptr, 0.0, Q.k(u), v2);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.stencil(r, w, nullptr, 0.0, k0, v2);
         v[0] = v2[0];
         v[1] = v2[1];
         v[2] = v2[0];
       } else {
         const float* uvec = (cheb & 1) ? A.zA : A.zB;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.apply_sums(uvec, r, w, Q.k(u), v);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.apply_sums(uvec, r, w, k0, v);
       }
       block_sum_f32<3>(v, wred, fsum);
       const double dv[3] = {(double)fsum[0], (double)fsum[1], (double)fsum[2]};
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       const float be = sc_beta * sc_pscale;
       const float* uvec = cheb == 1 ? r : ((cheb & 1) ? A.zA : A.zB);
       float v[1] = {0.0f};
-      for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) v[0] += ops.form(p, uvec, w, s, Q.k(u), be);
+      for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) v[0] += ops.form(p, uvec, w, s, k0, be);
       block_sum_f32<1>(v, wred, fsum);
       const double dv[1] = {(double)fsum[0]};
       publish(prow, NB, dv, 1);
@@ -403,19 +405,25 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       const float al = sc_alpha, be = sc_beta;
       const bool keep = sc_keep != 0;
       if (cheb == 1) {
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) ops.update(p, r, w, s, e, Q.k(u), al, be, keep);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) ops.update(p, r, w, s, e, k0, al, be, keep);
       } else {
         // the same update with u = M^-1 r
         const float* uvec = (cheb & 1) ? A.zA : A.zB;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x)
-          ops.update_u(p, uvec, r, w, s, e, Q.k(u), al, be, keep);
+        for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0)
+          ops.update_u(p, uvec, r, w, s, e, k0, al, be, keep);
       }
     }
     // the case's barrier (a case on one block needs only the block barrier: its own global
     // writes are visible to its threads after it)
     if (nbc == 1) __syncthreads();
     else if (!range_sync(ctl.bar, case_bar, (unsigned int)nbc, target)) { ok = false; break; }
-    // ---- after the barrier: the slot's sums, the scalars and the next slot
+    // ---- after the barrier: the next slot, or the slot's sums, the scalars and the next slot
+    if (sl == SL_UPDATE || sl == SL_CHEB || sl == SL_FOLD || (sl == SL_FRESH && cheb > 1)) {
+      if (sl == SL_UPDATE && threadIdx.x == 0) sc_fresh = 0;
+      step = sl == SL_CHEB ? step + 1 : 1;
+      sl = sl == SL_FOLD ? SL_RESID : step < cheb ? SL_CHEB : SL_APPLY;
+      continue;
+    }
     const bool sums3 = (sl == SL_RESID && last_part) || sl == SL_APPLY || (sl == SL_FRESH && cheb == 1);
     double t3[3] = {0.0, 0.0, 0.0};
     if (sums3) range_sum<3>(prow, NB, E.block0, nbc, t3, dsum);
@@ -425,9 +433,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       t3[0] = t1[0];
     }
     if (threadIdx.x == 0) {
-      if (sl == SL_FOLD) {
-        sc_slot = SL_RESID;
-      } else if (sl == SL_RESID && !last_part) {
+      if (sl == SL_RESID && !last_part) {
         sc_part = part + 1;
       } else if (sl == SL_RESID) {
         sc_part = 0;
@@ -451,26 +457,12 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
           sc_fresh = 1;
           sc_slot = SL_FRESH;
         }
-      } else if (sl == SL_FRESH && cheb > 1) {
-        sc_j = 1;
-        sc_slot = SL_CHEB;
-      } else if (sl == SL_CHEB) {
-        if (sc_j + 1 < cheb) sc_j += 1;
-        else sc_slot = SL_APPLY;
       } else if (sl == SL_FORM) {
         sc_alpha = sc_gfresh / (float)t3[0];
         sc_igamma = 1.0f / sc_gfresh;
         sc_ialpha = 1.0f / sc_alpha;
         sc_keep = 1;
         sc_slot = SL_UPDATE;
-      } else if (sl == SL_UPDATE) {
-        sc_fresh = 0;
-        if (cheb > 1) {
-          sc_j = 1;
-          sc_slot = SL_CHEB;
-        } else {
-          sc_slot = SL_APPLY;
-        }
       } else if (sums3) {
         // SL_APPLY, or SL_FRESH with Jacobi: gamma = (r, u), delta = (w, u), (r, r)
         const float gamma = (float)t3[0], delta = (float)t3[1], rr32 = (float)t3[2];
@@ -525,6 +517,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       }
     }
     __syncthreads();
+    sl = sc_slot;
   }
   if (lb == 0 && threadIdx.x == 0) {
     const bool conv = ok && sc_stop == 1;
