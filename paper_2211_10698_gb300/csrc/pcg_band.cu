@@ -39,7 +39,7 @@
 // What bounds it: the chain of one iteration, k + 1 block barriers, one L2 hop between SMs (907
 // cycles measured) and the scalars; on large tiles the instructions of the k + 1 passes.  Measured per
 // iteration against the best plan of pcg_mixed.cu and pcg_mixed1.cu: 1024x512, k = 3: 10.8 -> 7.4 us;
-// 2048x1024, k = 2: 27.5 -> 17.7 us; 701x333, Jacobi: 4.9 -> 4.1 us.
+// 2048x1024, k = 2: 27.5 -> 16.4 us; 701x333, Jacobi: 4.9 -> 4.1 us.
 #include <algorithm>
 
 #include "batch_common.cuh"
@@ -534,48 +534,67 @@ __device__ __forceinline__ int band_segment(const BandSolve& f, const int tile, 
     // while the sums go round: e += alpha p of the update above, and the band's w
     const unsigned int in = anew(rows_in), mo = anew(rows_own);
     const int wo = anew(woff);
-    if (PG) {
+    auto correct = [&]() {
+      if (PG) {
+        // three rows' p and e in flight at a time
 #pragma unroll
-      for (int q = 0; q < RS; ++q)
-        p[q] = own && ((mo >> q) & 1u) ? *reinterpret_cast<const float4*>(f.m.p + (wo + q * g.pitch)) : z4;
-    }
-    if (own) {
-      if (!fresh) {
+        for (int q0 = 0; q0 < RS; q0 += 3) {
+          float4 ev[3];
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            const int q = q0 + m < RS ? q0 + m : RS - 1;
+            if (q0 + m >= RS) continue;
+            const bool mine_q = own && ((mo >> q) & 1u);
+            p[q] = mine_q ? *reinterpret_cast<const float4*>(f.m.p + (wo + q * g.pitch)) : z4;
+            ev[m] = mine_q && !fresh ? *reinterpret_cast<const float4*>(f.E + (wo + q * g.pitch)) : z4;
+          }
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            const int q = q0 + m < RS ? q0 + m : RS - 1;
+            if (q0 + m < RS && own && ((mo >> q) & 1u) && !fresh)
+              *reinterpret_cast<float4*>(f.E + (wo + q * g.pitch)) = axpy4(ct.x, p[q], ev[m]);
+          }
+          row_end();
+        }
+      } else if (own && !fresh) {
 #pragma unroll
         for (int q = 0; q < RS; ++q)
           if ((mo >> q) & 1u) {
             float4* const ek = reinterpret_cast<float4*>(f.E + (wo + q * g.pitch));
             *ek = axpy4(ct.x, p[q], *ek);
-            if (q % 3 == 2) row_end();
           }
       }
-    }
+    };
+    // (many rows: the band's words first, before p takes registers: 2048x1024, k = 2, 17.7 -> 16.4 us
+    // per iteration; two or more rows' words in flight spill again, 17.3 us and more)
+    if (!PG) correct();
 #pragma unroll
     for (int q = 0; q < RS; ++q) {
-      if (!((in >> q) & 1u)) continue;
-      if (in_col && !(own && ((mo >> q) & 1u))) {
-        const unsigned long long* const k = WT + (wo + q * g.pitch);
-        unsigned long long w[4];
-        long long t0 = 0;
-        while (true) {
-          asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(k) : "memory");
-          asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[2]), "=l"(w[3]) : "l"(k + 2) : "memory");
-          if ((unsigned int)(w[0] >> 32) == tag && (unsigned int)(w[1] >> 32) == tag && (unsigned int)(w[2] >> 32) == tag &&
-              (unsigned int)(w[3] >> 32) == tag)
-            break;
-          if (t0 == 0) t0 = clock64();
-          else if (clock64() - t0 > f.m.d.bar.budget) {
-            atomicExch(f.m.d.bar.err, 1);
-            sh.fail = 1;
-            break;
-          }
+      if (!((in >> q) & 1u) || !in_col || (own && ((mo >> q) & 1u))) continue;
+      const unsigned long long* const k = WT + (wo + q * g.pitch);
+      unsigned long long w[4];
+      auto poll = [&]() {
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(k) : "memory");
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[2]), "=l"(w[3]) : "l"(k + 2) : "memory");
+      };
+      poll();
+      long long t0 = 0;
+      while ((unsigned int)(w[0] >> 32) != tag || (unsigned int)(w[1] >> 32) != tag || (unsigned int)(w[2] >> 32) != tag ||
+             (unsigned int)(w[3] >> 32) != tag) {
+        if (t0 == 0) t0 = clock64();
+        else if (clock64() - t0 > f.m.d.bar.budget) {
+          atomicExch(f.m.d.bar.err, 1);
+          sh.fail = 1;
+          break;
         }
-        const float4 v = make_float4(__uint_as_float((unsigned int)w[0]), __uint_as_float((unsigned int)w[1]),
-                                     __uint_as_float((unsigned int)w[2]), __uint_as_float((unsigned int)w[3]));
-        if (REG) wq[REG ? q : 0] = v;
-        else st(oW, q, v);
+        poll();
       }
+      const float4 v = make_float4(__uint_as_float((unsigned int)w[0]), __uint_as_float((unsigned int)w[1]),
+                                   __uint_as_float((unsigned int)w[2]), __uint_as_float((unsigned int)w[3]));
+      if (REG) wq[REG ? q : 0] = v;
+      else st(oW, q, v);
     }
+    if (PG) correct();
     __syncthreads();
     ct = sh.ctl;
     const int flow = __float_as_int(ct.z);
