@@ -474,6 +474,8 @@ ccm_status solve_poisson_mixed(ccm_case c, double* x, double* b) {
     launch_residual64(c->cv, g, x, b, c->fb, c->dpart, c->mixed_sums, st);
     CUDA_TRY(cudaMemcpyAsync(sums, c->mixed_sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
+    // b = 0: x = 0, whatever the warm start was
+    if (sums[1] == 0.0) CUDA_TRY(cudaMemsetAsync(x, 0, g.count() * sizeof(double), st));
     if (sums[1] == 0.0 || sums[0] <= c->cfg.tol_p * c->cfg.tol_p * sums[1]) { conv = true; break; }
     CUDA_TRY(cudaMemsetAsync(c->fx, 0, g.count() * sizeof(float), st));
     PoissonSolve<float> a{};
@@ -803,6 +805,11 @@ ccm_status case_mixed_residual(ccm_case c, double* host2) {
   CUDA_TRY(cudaMemcpyAsync(host2, c->mixed_sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   CUDA_TRY(cudaMemsetAsync(c->fx, 0, c->g.count() * sizeof(float), c->st));
   c->launches += 2;
+  return CCM_OK;
+}
+// b = 0: Phi = 0, whatever the warm start was
+ccm_status case_mixed_zero(ccm_case c) {
+  CUDA_TRY(cudaMemsetAsync(c->phi, 0, c->g.count() * sizeof(double), c->st));
   return CCM_OK;
 }
 void case_mixed_correct(ccm_case c) {

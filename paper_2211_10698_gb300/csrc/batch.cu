@@ -314,6 +314,10 @@ static ccm_status batch_mixed(ccm_batch b) {
       CaseSolveView v;
       case_solve_view(b->cases[i], &v);
       const double tolp = v.tol;
+      if (bb[i] == 0.0) {
+        ccm_status s = case_mixed_zero(b->cases[i]);
+        if (s != CCM_OK) return s;
+      }
       if (bb[i] == 0.0 || rr[i] <= tolp * tolp * bb[i]) {
         done[i] = 1;
         outer[i] = sweep;

@@ -449,6 +449,7 @@ void case_step_done(ccm_case c);
 void case_poisson_fp32(ccm_case c, PoissonSolve<float>* a);
 ccm_status case_mixed_project(ccm_case c, bool with_rhs);
 ccm_status case_mixed_residual(ccm_case c, double* host2);
+ccm_status case_mixed_zero(ccm_case c);  // Phi = 0
 void case_mixed_correct(ccm_case c);
 void case_mixed_account(ccm_case c, long long inner, int outer, double rr, double bb, bool converged);
 int* case_inner_iters_dev(ccm_case c);

@@ -285,6 +285,10 @@ __device__ __noinline__ int band_restart(const int tile, BandShared<NW>& sh, con
     if (sh.bb == 0.0 || sh.rr <= d.tol * d.tol * sh.bb) sh.stop = 1;
   }
   __syncthreads();
+  // b = 0: x = 0, whatever the warm start was (every block has read x before the barrier above)
+  if (sh.bb == 0.0)
+    for (int q = t; q < T.Ht * kRow; q += (NW + 1) * 32)
+      if (q % kRow < T.Wt) d.x[g.idx(T.i0 + q % kRow, T.j0 + q / kRow)] = 0.0;
   if (sh.stop != 0 || last) return 2;
   const double sig = sh.sigma;
   for (int ry = wid; ry < T.rows; ry += NW + 1) {

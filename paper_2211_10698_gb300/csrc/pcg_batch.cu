@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_sc_batch(const ScaledBatchEn
   }
   for (CellWalk cw(first, stride, ch.t1, nx); cw.ok(); cw.next()) {
     const size_t k = g.idx(cw.i, cw.j);
-    a.x[k] = a.isd[k] * xs[k];
+    a.x[k] = ok && sc_bb == 0.0 ? 0.0 : a.isd[k] * xs[k];  // b = 0: x = 0, whatever the warm start was
   }
   if (lb == 0 && threadIdx.x == 0) {
     const bool conv = ok && sc_stop == 1;
@@ -519,6 +519,9 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
     __syncthreads();
     sl = sc_slot;
   }
+  // b = 0: x = 0, whatever the warm start was (every block has read x before the case's last barrier)
+  if (ok && sc_bb == 0.0)
+    for (CellWalk cw(ch.t0 + (int)threadIdx.x, blockDim.x, ch.t1, nx); cw.ok(); cw.next()) d.x[g.idx(cw.i, cw.j)] = 0.0;
   if (lb == 0 && threadIdx.x == 0) {
     const bool conv = ok && sc_stop == 1;
     d.out.iters[0] = ok ? sc_it : 0;

@@ -189,11 +189,11 @@ __global__ void __launch_bounds__(kCT, 1) k_pcg_poisson_cluster(ClusterSolve f) 
       sc_den = sc_den_next;
     }
   }
-  // x = D^-1/2 x~ on the band
+  // x = D^-1/2 x~ on the band (0 for b = 0, whatever the warm start was)
   for (int l = threadIdx.x; l < ncell; l += kCT) {
     const int jl = l / nx, i = l - jl * nx;
     const size_t k = g.idx(i, j0 + jl);
-    a.x[k] = a.isd[k] * xs[l];
+    a.x[k] = sc_bb == 0.0 ? 0.0 : a.isd[k] * xs[l];
   }
   if (q == 0 && threadIdx.x == 0) {
     const bool conv = sc_stop == 1;

@@ -704,9 +704,11 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     cur = nxt;
   }
   if (sh.fail) ok = false;
+  // b = 0: the solution is 0, whatever the warm start was
+  const bool none = ok && sh.bb == 0.0;
   for (int q = 0; q < nq; ++q) {
     const size_t k = k0 + q * kstep;
-    a.x[k] = a.isd[k] * (RES ? sx[t + q * NT] : xs[k]);
+    a.x[k] = none ? 0.0 : a.isd[k] * (RES ? sx[t + q * NT] : xs[k]);
   }
   if (tile == 0 && t == 0) {
     const bool conv = ok && sh.stop == 1;

@@ -349,6 +349,9 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_pcg_poisson_mixed(MixedSolve
     fold(isig, false);
     if (!grid_sync(d.bar, target) || !residual64(false)) ok = false;
   }
+  // b = 0: x = 0, whatever the warm start was (every block has read x before residual64's barrier)
+  if (ok && sc_bb == 0.0)
+    for (CellWalk cw(first, stride, ch.t1, nx); cw.ok(); cw.next()) x[g.idx(cw.i, cw.j)] = 0.0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const bool conv = ok && sc_stop == 1;
     d.out.iters[0] = ok ? sc_it : 0;

@@ -526,6 +526,12 @@ __device__ __forceinline__ void mixed1_body(const Mixed1Solve& f) {
     fold(false);
     if (!grid_sync(d.bar, target) || !residual64(false)) ok = false;
   }
+  // b = 0: x = 0, whatever the warm start was (every block has read x before residual64's barrier)
+  if (ok && sc_bb == 0.0)
+    for (int q = threadIdx.x; q < nown; q += kNT) {
+      const int i = i0 + q % TX, j = j0 + q / TX;
+      if (i < i1 && j < j1) x[g.idx(i, j)] = 0.0;
+    }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const bool conv = ok && sc_stop == 1;
     d.out.iters[0] = ok ? sc_it : 0;
