@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "ccm_internal.cuh"
+#include "fused_plan.h"
 
 namespace ccm {
 
@@ -123,7 +124,6 @@ struct FusedSolve {
   int dcache;               // (resident) room for every cell's coefficients in shared memory
   int defer;                // (resident) a second r frame, so that p waits for the barrier as x does
 };
-constexpr int kFusedTilesMax = 512;  // tiles of a launch, at most (two per SM)
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
 // One case of a batched launch of resident tiles: its first block (one block per tile).
 struct FusedBatchEntry {
@@ -135,13 +135,8 @@ struct FusedBatchEntry {
 size_t fused_batch_plan(FusedSolve* f, int blocks);
 int fused_batch_blocks();    // blocks of such a launch, at most
 size_t fused_batch_cells();  // no tile of one has more cells
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells = 512, int max_tx = 512);
 int fused_blocks();
-size_t fused_resident_smem_min(int TX, int TY);
 bool fused_resident_ok(int TX, int TY, int ntiles);
-// Mailbox slots of a resident plan, and of any resident plan of a grid.
-size_t fused_mail_slots(int nx, int TX, int TY, int ntiles);
-size_t fused_mail_slots_max(int nx, int ny);
 
 // The same solve for small grids inside one thread-block cluster (pcg_cluster.cu).
 struct ClusterSolve {

@@ -9,8 +9,10 @@
 // lives in one file-scope __device__ array of fixed size instead of memory the library
 // allocates.  The kernel is the resident one-barrier solve (pcg_fused.cu) in its built-in plan:
 // a tile's vectors stay in shared memory, so the array holds the right-hand side, the first
-// residual and the mailboxes of the tiles (every grid within the limit fits: at most 863 cells
-// per SM).  A singular case (no outflow side) projects onto zero mean at the start and the end.
+// residual and the mailboxes of the tiles.  Every grid within the limit has such a plan
+// (tests/test_fused_plan.py goes through them all); where the smallest tiles are wide and flat
+// their rings would not fit the mailboxes, and the plan takes narrower or taller ones (500x150:
+// 150 tiles of 256x2 instead of 512x1).  A singular case (no outflow side) projects onto zero mean at the start and the end.
 // The caller passes the right-hand side and the solution in device memory of its own.
 //
 // The array (about 6.4 MB) stays resident on every GPU that loads the library until the

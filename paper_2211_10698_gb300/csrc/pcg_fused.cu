@@ -748,30 +748,6 @@ __global__ void __launch_bounds__(NT + 32, MINB) k_fused_batch(const FusedBatchE
 
 }  // namespace
 
-// Tile shape for at most `blocks` blocks: TX a power of two in 32..max_tx, as many tile rows as
-// the blocks allow while a tile keeps about min_cells cells; the shape with the smallest
-// largest tile wins (then the shortest ring).  One block per tile.
-void fused_tiles(int nx, int ny, int blocks, int* TX, int* TY, int* nbx, int* ntiles, int min_cells, int max_tx) {
-  long long best = -1, best_ring = 0;
-  for (int tx = 32; tx <= max_tx; tx *= 2) {
-    const int bxn = (nx + tx - 1) / tx;
-    if (bxn > blocks) continue;
-    const int wx = std::min(tx, nx);
-    const int min_ty = (min_cells + wx - 1) / wx;
-    const int byn = std::max(1, std::min(blocks / bxn, (ny + min_ty - 1) / min_ty));
-    const int ty = (ny + byn - 1) / byn;
-    const long long cells = (long long)wx * ty, ring = 2LL * (wx + ty);
-    if (best < 0 || cells < best || (cells == best && ring < best_ring)) {
-      best = cells;
-      best_ring = ring;
-      *TX = tx;
-      *TY = ty;
-      *nbx = bxn;
-      *ntiles = bxn * ((ny + ty - 1) / ty);
-    }
-  }
-}
-
 constexpr size_t kFusedSmemMax = 64 * 1024;  // f1: ring and list of non-uniform cells, per block
 
 namespace {
@@ -783,17 +759,6 @@ int sm_count() {
   return sms;
 }
 
-// Computing threads of a plan's blocks, the same whether its tiles are resident or not (so that
-// both run the same additions in the same order): one or two cells per thread on small tiles,
-// whose iteration is paced by its barriers and block sums; 512 where the FP64 pipe sets the pace;
-// 256 where two blocks of an SM share it (their threads then have registers enough).
-int fused_threads(int TX, int TY, int ntiles, int sms) {
-  const int cells = TX * TY;
-  if (cells <= 256 && TX <= 128) return 128;
-  if (TX <= 256 && (cells <= 1024 || (ntiles > sms && cells <= 2048))) return 256;
-  return 512;
-}
-
 const void* fused_kernel(bool resident, int nt, bool two) {
   if (nt == 128) return resident ? (const void*)k_pcg_poisson_f2<128, 2> : (const void*)k_pcg_poisson_f1<128, 2>;
   if (!resident) return nt == 256 ? (const void*)k_pcg_poisson_f1<256, 2> : (const void*)k_pcg_poisson_f1<512, 2>;
@@ -801,22 +766,12 @@ const void* fused_kernel(bool resident, int nt, bool two) {
   return two ? (const void*)k_pcg_poisson_f2<512, 2> : (const void*)k_pcg_poisson_f2<512, 1>;
 }
 
-// Dynamic shared memory of a tile with its vectors resident (f2): x~, p, s, w, r~ with its
-// one-cell frame (two of them with `defer`), the ring's s, the coefficients of every cell
-// (`dcache`) or of nt listed cells (`lcache`), a list of up to one entry per cell.
-size_t resident_smem(int TX, int TY, int nt, bool dcache, bool defer, bool lcache) {
-  const size_t txy = (size_t)TX * (size_t)TY;
-  return sizeof(double) * (4 * txy + (defer ? 2 : 1) * ((size_t)TX + 2) * ((size_t)TY + 2) +
-                           2 * ((size_t)TX + (size_t)TY) + (dcache ? 5 * txy : 0) + (lcache ? 5 * (size_t)nt : 0)) +
-         sizeof(int) * txy;
-}
-
 // Shared memory of ntiles resident tiles of TX x TY cells, which must fit the GPU at once: with
 // every cell's coefficients cached, with a second r frame (defer) and with the listed cells'
 // coefficients cached where they fit too; 0 if nothing fits.
 size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
   const int sms = sm_count(), nt = fused_threads(TX, TY, ntiles, sms);
-  if (ntiles < 1 || ntiles > 2 * sms || TX * TY > 32 * nt) return 0;
+  if (ntiles < 1 || ntiles > 2 * sms || TX * TY > kFusedRows * nt) return 0;
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -853,31 +808,7 @@ int fused_blocks() {
   return sm_count() * per;
 }
 
-size_t fused_resident_smem_min(int TX, int TY) { return resident_smem(TX, TY, 0, false, false, false); }
-
 bool fused_resident_ok(int TX, int TY, int ntiles) { return resident_shape(TX, TY, ntiles, nullptr) != 0; }
-
-size_t fused_mail_slots(int nx, int TX, int TY, int ntiles) {
-  return (size_t)2 * (size_t)ntiles * 2 * (size_t)(TY + std::min(TX, nx));
-}
-
-// The most slots any resident plan of a grid can need: every tile width, every count of tile
-// rows up to kFusedTilesMax tiles whose smallest tile could stay in shared memory.
-size_t fused_mail_slots_max(int nx, int ny) {
-  size_t most = 0;
-  for (int tx = 32; tx <= 512; tx *= 2) {
-    const int bxn = (nx + tx - 1) / tx;
-    for (int byn = 1; byn <= ny && (long long)bxn * byn <= kFusedTilesMax; ++byn) {
-      const int ty = (ny + byn - 1) / byn;
-      if (fused_resident_smem_min(tx, ty) > 227 * 1024) continue;
-      most = std::max(most, fused_mail_slots(nx, tx, ty, bxn * ((ny + ty - 1) / ty)));
-    }
-  }
-  return most;
-}
-
-// Cells of a built-in resident tile, at least about.
-constexpr int kResidentCells = 128;
 
 // Batched launch: two blocks of 256 computing threads per SM.  Blocks of different cases share an
 // SM, and one's vectors fill the FP64 pipe while the other waits for its reduction.
@@ -901,7 +832,7 @@ size_t fused_batch_cells() { return batch_room() / (5 * sizeof(double) + sizeof(
 size_t fused_batch_plan(FusedSolve* f, int blocks) {
   f->ntiles = 0;
   fused_tiles(f->a.g.nx, f->a.g.ny, blocks, &f->TX, &f->TY, &f->nbx, &f->ntiles, kResidentCells, kBatchNT);
-  if (f->ntiles < 1 || f->ntiles > blocks || f->TX * f->TY > 32 * kBatchNT) return 0;
+  if (f->ntiles < 1 || f->ntiles > blocks || f->TX * f->TY > kFusedRows * kBatchNT) return 0;
   if (f->mail_slots < fused_mail_slots(f->a.g.nx, f->TX, f->TY, f->ntiles)) return 0;
   f->resident = 1;
   f->wx = std::min(f->TX, f->a.g.nx);
@@ -932,10 +863,11 @@ cudaError_t run_fused_batch(const FusedBatchEntry* dev_cases, const int* dev_blo
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   const int blocks = fused_blocks(), sms = sm_count();
   if (f.TX == 0) {
-    // the built-in plan: resident tiles, one per SM, where they fit, else two in global memory
-    fused_tiles(f.a.g.nx, f.a.g.ny, sms, &f.TX, &f.TY, &f.nbx, &f.ntiles, kResidentCells);
-    const bool fits = resident_shape(f.TX, f.TY, f.ntiles, nullptr) != 0 && f.mail &&
-                      f.mail_slots >= fused_mail_slots(f.a.g.nx, f.TX, f.TY, f.ntiles);
+    // the built-in plan: resident tiles, one per SM, where they and their mailboxes fit, else two in
+    // global memory
+    fused_tiles(f.a.g.nx, f.a.g.ny, sms, &f.TX, &f.TY, &f.nbx, &f.ntiles, kResidentCells, 512,
+                f.mail ? f.mail_slots : SIZE_MAX);
+    const bool fits = f.mail && resident_shape(f.TX, f.TY, f.ntiles, nullptr) != 0;
     if (!fits && f.resident) return cudaErrorInvalidConfiguration;  // the caller has resident tiles only
     if (!fits) fused_tiles(f.a.g.nx, f.a.g.ny, blocks, &f.TX, &f.TY, &f.nbx, &f.ntiles);
     f.resident = fits ? 1 : 0;
