@@ -97,6 +97,23 @@ struct ScaledSolve {
   PcgOut out;
 };
 
+// Dynamic shared memory that a launch of `kernel` may ask for, at most, and leave to ask for it
+// (0 on an error).  The limit belongs to the kernel on its device and not to a launch: always set to
+// the same value, it is right for every thread whatever the others launch.
+inline size_t allow_most_smem(const void* kernel) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes at{};
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&at, kernel) != cudaSuccess || (size_t)optin <= at.sharedSizeBytes ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)at.sharedSizeBytes) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (size_t)optin - at.sharedSizeBytes;
+}
+
 // The same solve with one grid barrier per iteration (pcg_fused.cu): 2-D tiles, the ring of
 // each tile recomputed by its block, r, w, s double-buffered.  a.xs and a.p are used, a.r,
 // a.w, a.s are not.

@@ -906,8 +906,7 @@ cudaError_t run_poisson_band(BandSolve f, cudaStream_t st) {
   if (!band_fits(&f)) return cudaErrorInvalidConfiguration;
   const BandShape& shape = kShapes[f.shape];
   const size_t smem = band_smem(f.TY, f.m.cheb) + kSlot * (size_t)(f.ncut - 2);
-  cudaError_t e = cudaFuncSetAttribute(shape.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (smem > allow_most_smem(shape.kernel)) return cudaErrorInvalidConfiguration;
   cudaMemsetAsync(f.m.d.bar.count, 0, sizeof(unsigned int) * kBarWords, st);
   void* params[] = {&f};
   return cudaLaunchCooperativeKernel(shape.kernel, f.ntiles, shape.nw * 32 + 32, params, smem, st);

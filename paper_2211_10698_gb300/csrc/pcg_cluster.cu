@@ -221,8 +221,9 @@ cudaError_t run_poisson_cluster(ClusterSolve f, int C, cudaStream_t st) {
   f.nmax = (g.ny + C - 1) / C * g.nx;
   const size_t smem = cluster_smem_bytes(g.nx, g.ny, C);
   if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(k_pcg_poisson_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && C > 8)
+  if (smem > allow_most_smem((const void*)k_pcg_poisson_cluster)) return cudaErrorInvalidConfiguration;
+  cudaError_t e = cudaSuccess;
+  if (C > 8)
     e = cudaFuncSetAttribute(k_pcg_poisson_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -772,17 +772,14 @@ const void* fused_kernel(bool resident, int nt, bool two) {
 size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
   const int sms = sm_count(), nt = fused_threads(TX, TY, ntiles, sms);
   if (ntiles < 1 || ntiles > 2 * sms || TX * TY > kFusedRows * nt) return 0;
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const void* kern = fused_kernel(true, nt, ntiles > sms);
+  const size_t room = allow_most_smem(kern);
   for (int k = 7; k >= 0; --k) {
     const bool dc = (k & 4) != 0, df = (k & 2) != 0, lc = (k & 1) != 0;
     const size_t smem = resident_smem(TX, TY, nt, dc, df, lc);
-    if (smem > (size_t)optin) continue;
+    if (smem > room) continue;
     int per = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nt + 32, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nt + 32, smem) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -802,7 +799,7 @@ size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
 int fused_blocks() {
   const void* kern = fused_kernel(false, 512, true);
   int per = 0;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
+  allow_most_smem(kern);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 512 + 32, kFusedSmemMax);
   per = per > 2 ? 2 : (per < 1 ? 1 : per);
   return sm_count() * per;
@@ -853,8 +850,7 @@ cudaError_t run_fused_batch(const FusedBatchEntry* dev_cases, const int* dev_blo
                             size_t smem, cudaStream_t st) {
   if (!ctl.case_bar || ctl.ncases < 1) return cudaErrorInvalidValue;
   const void* kern = (const void*)k_fused_batch<kBatchNT, kBatchPerSM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (smem > allow_most_smem(kern)) return cudaErrorInvalidConfiguration;
   cudaMemsetAsync(ctl.case_bar, 0, sizeof(unsigned int) * kCaseBarStride * (size_t)ctl.ncases, st);
   void* params[] = {(void*)&dev_cases, (void*)&dev_block_case};
   return cudaLaunchCooperativeKernel(kern, blocks, kBatchNT + 32, params, smem, st);
@@ -889,7 +885,7 @@ cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
     // the list of non-uniform cells takes what is left, up to one entry per tile cell
     f.list_cap = (int)std::min<size_t>((kFusedSmemMax - ring) / sizeof(int), (size_t)f.TX * (size_t)f.TY);
     smem = ring + sizeof(int) * (size_t)f.list_cap;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
+    if (smem > allow_most_smem(kernel)) return cudaErrorInvalidConfiguration;
   }
   cudaMemsetAsync(f.a.bar.count, 0, sizeof(unsigned int) * kBarWords, st);
   void* params[] = {&f};

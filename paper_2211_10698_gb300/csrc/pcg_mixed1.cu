@@ -553,12 +553,9 @@ __global__ void __launch_bounds__(kNT, 1) k_pcg_poisson_m2(const __grid_constant
 }
 
 int mixed1_per_sm(size_t smem, int resident) {
-  int dev = 0, per = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  int per = 0;
   const void* kern = resident ? (const void*)k_pcg_poisson_m2 : (const void*)k_pcg_poisson_m1;
-  if (smem > (size_t)optin ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (smem > allow_most_smem(kern) ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kNT, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
