@@ -142,6 +142,7 @@ struct FusedSolve {
   int defer;                // (resident) a second r frame, so that p waits for the barrier as x does
 };
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
+const void* fused_global_kernel(int nt);  // tiles in global memory, nt threads per block (pcg_fused_global.cu)
 // One case of a batched launch of resident tiles: its first block (one block per tile).
 struct FusedBatchEntry {
   FusedSolve f;

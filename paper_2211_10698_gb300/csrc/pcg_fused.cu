@@ -7,36 +7,32 @@
 // itself, from the previous iteration's vectors:
 //     r_{i+1} = r_i - alpha_i (w_i + beta_i s_{i-1})      (= r_i - alpha_i s_i),
 // so the stencil needs no other block's work of the same iteration and only the reduction
-// needs a barrier.  r, w and s are double-buffered by iteration parity: iteration i reads
-// buffer i%2 everywhere and writes buffer (i+1)%2 for its own cells, so the ring cells a
-// neighbouring block reads are never the ones being written.
+// needs a barrier.
 //
-// Per iteration, in each block:
-//   1. own cells: s_i, p_i, x~ += alpha p_i, r_{i+1} (written to the next buffers);
-//      ring cells: r_{i+1} into shared memory (zero outside the domain)
-//   2. block barrier; own cells: w_{i+1} = K~ r_{i+1} (neighbours inside the tile from the
-//      next buffer, on the ring from shared memory), the sums; block sum; grid barrier
-//   3. every block sums the partials in the same order and forms the scalars.
+// Two kernels run this iteration: k_pcg_poisson_f1 (pcg_fused_global.cu) keeps the vectors in global
+// memory; k_pcg_poisson_f2 here keeps its tile's x~, r, p, s and w in shared memory for the whole
+// solve.  Per iteration, in each block of f2:
+//   1. own cells: s_i, r_{i+1}; ring cells: r_{i+1}, in the frame of the tile's r (zero outside the
+//      domain)
+//   2. block barrier; own cells: w_{i+1} = K~ r_{i+1} and the sums; the grid barrier
+//   3. every block forms the scalars from the same sums.
 // With one barrier per iteration a block can publish the next iteration's partials while a
 // slower block still reads this iteration's, so the partials alternate between two sets of
 // rows by iteration parity.
 // Tiles are TX x TY cells (TX a power of two, 32..512), one per block; the host picks the
-// shape that makes the largest tile smallest.
+// shape that makes the largest tile smallest (fused_plan.h).
 //
-// Two instantiations of the same iteration: k_pcg_poisson_f1 keeps x~, r, p, s and w in global
-// memory (L2) and publishes r, w and s there; k_pcg_poisson_f2 keeps its tile's x~, r, p, s, w
-// and row kinds in shared memory for the whole solve.  f2's ring needs one value per cell and
-// iteration from the neighbours: w.  The ring's r and s are kept by the tile that reads them,
-// updated with the same recurrences as their owner's (equal bit for bit), so a tile pushes the w
-// of its perimeter into its neighbours' mailboxes (one 16-byte slot per ring cell holding the
-// value and the iteration's number, double-buffered by parity) and reads its own mailbox.  The
-// slot's tag says that the value is there, and the words of the reduction carry the sums, so no
-// release or acquire, and no wait for outstanding stores, is left in f2's iteration.
+// f2's ring needs one value per cell and iteration from the neighbours: w.  The ring's r and s are
+// kept by the tile that reads them, updated with the same recurrences as their owner's (equal bit
+// for bit), so a tile pushes the w of its perimeter into its neighbours' mailboxes (one 16-byte slot
+// per ring cell holding the value and the iteration's number, double-buffered by parity) and reads
+// its own mailbox.  The slot's tag says that the value is there, and the words of the reduction carry
+// the sums, so no release or acquire, and no wait for outstanding stores, is left in the iteration.
 //
 // One further warp per block (the communication warp) sums the block's digits, adds them to the
 // reduction's words, waits for the grid's and forms the scalars of the next iteration in integer
 // arithmetic (pcg_scalar.cuh), while the other warps do the work that no other block reads:
-// p = r_i + beta p and x~ += alpha p (f2; r_i is kept beside r_{i+1} in a second framed copy,
+// p = r_i + beta p and x~ += alpha p (r_i is kept beside r_{i+1} in a second framed copy,
 // where the tile leaves room for it: otherwise p is formed in step 1 and only x~ waits), and the
 // wait for the ring's next w.  The FP64 pipe (one warp instruction per 64 cycles on each
 // sub-partition) stays with the vectors, and the serial chain beside it.
@@ -84,14 +80,12 @@ __device__ __forceinline__ void digits_ready(bool wait) {
 }
 
 // One tile of a solve: tile `tile` of the case's f.ntiles, one block of NT + 32 threads each.
-// RES: the tile's vectors live in shared memory (f2); otherwise in global memory (f1).
-template <bool RES, int NT>
+template <int NT>
 __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, FusedShared<NT>& sh) {
-  // dynamic shared memory: with RES x~, p, s, w of the tile (TX*TY each), r~ of the tile in a
-  // one-cell frame ((TX+2)*(TY+2), the frame holding the ring), with f.defer twice, then the
-  // ring's s [W: TY][E: TY][S: TX][N: TX] (without RES: the ring's r), then with RES and f.dcache
-  // the five scaled coefficients of every cell, with RES and f.lcache those of the first NT listed
-  // cells, then the list
+  // dynamic shared memory: x~, p, s, w of the tile (TX*TY each), r~ of the tile in a one-cell
+  // frame ((TX+2)*(TY+2), the frame holding the ring), with f.defer twice, then the ring's s
+  // [W: TY][E: TY][S: TX][N: TX], then with f.dcache the five scaled coefficients of every cell,
+  // with f.lcache those of the first NT listed cells, then the list
   extern __shared__ double dyn[];
   unsigned int target = 0;
   const ScaledSolve& a = f.a;
@@ -111,22 +105,22 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   const int nq = !comm && ci < i1 && j0 + ty0 < j1 ? (j1 - j0 - ty0 + RP - 1) / RP : 0;
   const size_t k0 = g.idx(ci, j0 + ty0);  // of own cell 0 (used where nq > 0)
   const size_t kstep = (size_t)RP * P;
-  double* const sx = dyn;  // the RES arrays (unused otherwise)
+  double* const sx = dyn;
   double* const sp = dyn + TXY;
   double* const ss = dyn + 2 * TXY;
   double* const sw = dyn + 3 * TXY;
-  // RES: r~ of the tile with a one-cell frame that holds the ring, so that the stencil reads
-  // every neighbour from one array without a branch; with defer two of them alternate
+  // r~ of the tile with a one-cell frame that holds the ring, so that the stencil reads every
+  // neighbour from one array without a branch; with defer two of them alternate
   const int TXP = TX + 2, FR = TXP * (TY + 2);
   const int lp0 = (ty0 + 1) * TXP + tx + 1, lpstep = RP * TXP;  // frame index of own cell 0, and step
-  const bool defer = RES && f.defer != 0;
+  const bool defer = f.defer != 0;
   double* sr = dyn + 4 * TXY;                         // r_i
   double* srn = defer ? sr + FR : sr;                 // r_{i+1}
-  double* const ring = RES ? dyn + 4 * TXY + (defer ? 2 : 1) * FR : dyn;
+  double* const ring = dyn + 4 * TXY + (defer ? 2 : 1) * FR;
   double* const dcoef = ring + 2 * (TX + TY);
-  double* const lcoef = dcoef + (RES && f.dcache ? 5 * TXY : 0);
-  int* const list = reinterpret_cast<int*>(lcoef + (RES && f.lcache ? 5 * NT : 0));
-  // index of cell (i, j) of the tile or its frame in the framed r~ (RES)
+  double* const lcoef = dcoef + (f.dcache ? 5 * TXY : 0);
+  int* const list = reinterpret_cast<int*>(lcoef + (f.lcache ? 5 * NT : 0));
+  // index of cell (i, j) of the tile or its frame in the framed r~
   auto lpad = [&](int i, int j) -> int { return (j - j0 + 1) * TXP + (i - i0 + 1); };
   // ring cells: W and E columns, then S and N rows, taken by threads t, t + NT, ...
   const int nring = 2 * (j1 - j0) + 2 * (i1 - i0);
@@ -144,7 +138,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   const bool my_ring = !comm && t < nring;
   const bool my_in = my_ring && ring_cell(t, my_ri, my_rj, my_slot);
   const int my_lp = lpad(my_ri, my_rj);
-  // RES: the mailbox, f.mail[parity][tile][slot]; nslot slots per tile (f.wx: the tile's width
+  // the mailbox, f.mail[parity][tile][slot]; nslot slots per tile (f.wx: the tile's width
   // clipped to the grid's)
   const int nslot = 2 * (TY + f.wx);
   auto mailbox = [&](int parity, int q) -> ulonglong2* { return f.mail + ((size_t)parity * nb + q) * nslot; };
@@ -168,38 +162,17 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   const double* __restrict__ cvs = a.cvs;
   const double* __restrict__ sd = a.sd;
   const double ax = a.ax, ay = a.ay, dreg = a.dreg;
-  double* __restrict__ xs = a.xs;
-  double* __restrict__ p = a.p;
   auto sync_grid = [&]() -> bool { return range_sync(a.bar, a.bar.count, (unsigned int)nb, target); };
 
-  // r~ at neighbour (i, j) of an own cell after step 1 (without RES): inside the tile from the
-  // next buffer, on the ring from shared memory
-  auto rnb = [&](const double* rn, int i, int j) -> double {
-    if (i < i0) return ring[j - j0];
-    if (i >= i1) return ring[TY + (j - j0)];
-    if (j < j0) return ring[2 * TY + (i - i0)];
-    if (j >= j1) return ring[2 * TY + f.wx + (i - i0)];
-    return rn[g.idx(i, j)];
-  };
   // r~ of own cell (i, j) and its neighbours after step 1
-  auto gather = [&](const double* rn, int i, int j, double (&r)[5]) {
-    if constexpr (RES) {
-      const double* q = srn + lpad(i, j);
-      r[0] = q[0]; r[1] = q[-1]; r[2] = q[1]; r[3] = q[-TXP]; r[4] = q[TXP];
-    } else {
-      r[0] = rn[g.idx(i, j)];
-      r[1] = rnb(rn, i - 1, j); r[2] = rnb(rn, i + 1, j); r[3] = rnb(rn, i, j - 1); r[4] = rnb(rn, i, j + 1);
-    }
+  auto gather = [&](int i, int j, double (&r)[5]) {
+    const double* q = srn + lpad(i, j);
+    r[0] = q[0]; r[1] = q[-1]; r[2] = q[1]; r[3] = q[-TXP]; r[4] = q[TXP];
   };
-  // w~ of own cell (i, j), tile-local index l, into the tile (RES, which also sends the
-  // perimeter's to the neighbours) or into wn
-  auto wput = [&](double* wn, int parity, unsigned int tag, int i, int j, int l, double wk) {
-    if constexpr (RES) {
-      sw[l] = wk;
-      if (i == i0 || i == i1 - 1 || j == j0 || j == j1 - 1) push(parity, tag, i - i0, j - j0, wk);
-    } else {
-      wn[g.idx(i, j)] = wk;
-    }
+  // w~ of own cell (i, j), tile-local index l, into the tile, the perimeter's also to the neighbours
+  auto wput = [&](int parity, unsigned int tag, int i, int j, int l, double wk) {
+    sw[l] = wk;
+    if (i == i0 || i == i1 - 1 || j == j0 || j == j1 - 1) push(parity, tag, i - i0, j - j0, wk);
   };
   // Rows of cut cells and rows next to a Neumann side (kind 2) are listed per tile, in a fixed
   // order, at the start.  The stencil pass applies the constant stencil to every own cell, so
@@ -212,7 +185,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   // small tile, of a few rows per thread, with any listed cell); and where the list does not hold
   // them.  (The scaled coefficient arrays hold the constants on uniform rows and zeros on inactive
   // ones.)
-  unsigned int m_in = 0u, m_list = 0u;  // RES: bit q: own cell q is inactive, is listed (nq <= 32)
+  unsigned int m_in = 0u, m_list = 0u;  // bit q: own cell q is inactive, is listed (nq <= 32)
   int nlist = 0;
   bool dense = false;
   {
@@ -220,10 +193,8 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     for (int q = 0; q < nq; ++q) {
       const int8_t km = kinds[k0 + q * kstep];
       mine += km == 2;
-      if (RES) {
-        m_in |= (km == 0 ? 1u : 0u) << q;
-        m_list |= (km == 2 ? 1u : 0u) << q;
-      }
+      m_in |= (km == 0 ? 1u : 0u) << q;
+      m_list |= (km == 2 ? 1u : 0u) << q;
     }
     // exclusive scan of the counts over the block (thread order)
     int incl = mine;
@@ -274,7 +245,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     const int8_t km = kinds[k];
     c[4] = (km == 1 ? dreg : (km == 2 ? sd[k] * sd[k] : 1.0)) - dreg;
   };
-  if constexpr (RES) {
+  {
     double c[5];
     if (dense && f.dcache)
       for (int q = 0, l = t; q < nq; ++q, l += NT) {
@@ -297,83 +268,57 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     v[2] += wk * r[0];
     return wk;
   };
-  // step 2 on own cells: w = K~ r (r in buffer rn, or the tile with RES), sums into v
-  auto stencil = [&](const double* rn, double* wn, int parity, unsigned int tag, double (&v)[4]) {
+  // step 2 on own cells: w = K~ r, sums into v
+  auto stencil = [&](int parity, unsigned int tag, double (&v)[4]) {
     double r[5], c[5];
     if (dense) {
       for (int q = 0, l = t; q < nq; ++q, l += NT) {
         const int j = j0 + ty0 + q * RP;
-        gather(rn, ci, j, r);
-        if (RES && f.dcache) {
+        gather(ci, j, r);
+        if (f.dcache) {
 #pragma unroll
           for (int e = 0; e < 5; ++e) c[e] = dcoef[e * TXY + l];
         } else {
           coefs(k0 + q * kstep, c);
         }
-        wput(wn, parity, tag, ci, j, l, row(r, c, v));
+        wput(parity, tag, ci, j, l, row(r, c, v));
       }
       return;
     }
     // the listed cells first: their chains of FP64 operations interleave with the other warps'
     // constant-stencil passes instead of trailing them
     if (q_l >= 0) {
-      gather(rn, q_i, q_j, r);
-      if (RES && f.lcache) {
+      gather(q_i, q_j, r);
+      if (f.lcache) {
 #pragma unroll
         for (int e = 0; e < 5; ++e) c[e] = lcoef[e * NT + t];
       } else {
         coefs(g.idx(q_i, q_j), c);
       }
-      wput(wn, parity, tag, q_i, q_j, q_l, row(r, c, v));
+      wput(parity, tag, q_i, q_j, q_l, row(r, c, v));
     }
     for (int q = myq + NT; q < nlist; q += NT) {
       const int l = list[q], i = i0 + l % TX, j = j0 + l / TX;
-      gather(rn, i, j, r);
+      gather(i, j, r);
       coefs(g.idx(i, j), c);
-      wput(wn, parity, tag, i, j, l, row(r, c, v));
+      wput(parity, tag, i, j, l, row(r, c, v));
     }
     // constant stencil on every own cell; the listed ones add nothing to the sums and are not
     // stored (selects and predicates: a branch would run the FP64 instructions of both sides)
-    if constexpr (RES) {
-      const double* z = srn + lp0;
+    const double* z = srn + lp0;
 #pragma unroll 2
-      for (int q = 0; q < nq; ++q, z += lpstep) {
-        const bool listed = (m_list >> q) & 1u;
-        const double rc = z[0];
-        double wk = rc - ax * (z[-1] + z[1]) - ay * (z[-TXP] + z[TXP]);
-        if ((m_in >> q) & 1u) wk = 0.0;
-        const double rs = listed ? 0.0 : rc;
-        v[0] += rs * rs;
-        v[2] += wk * rs;
-        if (!listed) {
-          sw[t + q * NT] = wk;
-          const int jr = ty0 + q * RP;
-          if (edge_col || jr == 0 || jr == hj_) push(parity, tag, tx, jr, wk);
-        }
-      }
-    } else {
-      for (int q = 0; q < nq; q += 2) {
-        const bool two = q + 1 < nq;
-        const int j = j0 + ty0 + q * RP, jb = two ? j + RP : j;
-        const size_t ka = k0 + q * kstep, kb = two ? ka + kstep : ka;
-        const int8_t kma = kinds[ka], kmb = kinds[kb];
-        double ra[5], rb[5];
-        gather(rn, ci, j, ra);
-        gather(rn, ci, jb, rb);
-        const double wa = kma == 0 ? 0.0 : ra[0] - ax * (ra[1] + ra[2]) - ay * (ra[3] + ra[4]);
-        if (kma != 2) {
-          wn[ka] = wa;
-          v[0] += ra[0] * ra[0];
-          v[2] += wa * ra[0];
-        }
-        if (two) {
-          const double wb = kmb == 0 ? 0.0 : rb[0] - ax * (rb[1] + rb[2]) - ay * (rb[3] + rb[4]);
-          if (kmb != 2) {
-            wn[kb] = wb;
-            v[0] += rb[0] * rb[0];
-            v[2] += wb * rb[0];
-          }
-        }
+    for (int q = 0; q < nq; ++q, z += lpstep) {
+      const bool listed = (m_list >> q) & 1u;
+      const double rc = z[0];
+      double wk = rc - ax * (z[-1] + z[1]) - ay * (z[-TXP] + z[TXP]);
+      if ((m_in >> q) & 1u) wk = 0.0;
+      const double rs = listed ? 0.0 : rc;
+      v[0] += rs * rs;
+      v[2] += wk * rs;
+      if (!listed) {
+        sw[t + q * NT] = wk;
+        const int jr = ty0 + q * RP;
+        if (edge_col || jr == 0 || jr == hj_) push(parity, tag, tx, jr, wk);
       }
     }
   };
@@ -407,28 +352,20 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
       const bool inactive = kinds[k] == 0;  // identity row: x = b exactly
       const double rk = inactive ? 0.0 : bk - K(a.x, k);
       const double x0 = inactive ? bk : sd[k] * a.x[k], r0 = a.isd[k] * rk;
-      if constexpr (RES) {
-        const int l = t + q * NT, jr = ty0 + q * RP;
-        sx[l] = x0;
-        srn[lp0 + q * lpstep] = r0;
-        ss[l] = 0.0;
-        sp[l] = 0.0;
-        if (edge_col || jr == 0 || jr == hj_) f.R[0][k] = r0;  // the neighbours' first ring
-      } else {
-        xs[k] = x0;
-        f.R[0][k] = r0;
-        f.S[0][k] = 0.0;
-        p[k] = 0.0;
-      }
+      const int l = t + q * NT, jr = ty0 + q * RP;
+      sx[l] = x0;
+      srn[lp0 + q * lpstep] = r0;
+      ss[l] = 0.0;
+      sp[l] = 0.0;
+      if (edge_col || jr == 0 || jr == hj_) f.R[0][k] = r0;  // the neighbours' first ring
       v[3] += bk * bk;
     }
   }
   // the fixed-point words and the mailboxes start at zero (they hold an earlier launch's); the
   // barriers of phase 0 order this before their first use
   if (tile == 0 && t < 2 * kFxWords) f.fxacc[(size_t)t * kFxStride] = 0ULL;
-  if constexpr (RES)
-    for (int q = t; q < 2 * nslot; q += NT + 32)
-      mailbox(q >= nslot, tile)[q >= nslot ? q - nslot : q] = make_ulonglong2(0ULL, 0ULL);
+  for (int q = t; q < 2 * nslot; q += NT + 32)
+    mailbox(q >= nslot, tile)[q >= nslot ? q - nslot : q] = make_ulonglong2(0ULL, 0ULL);
   bool ok = sync_grid();
   if (ok) {
     // w_0 = K~ r_0: every neighbour's r_0 is complete, read through the same ring path
@@ -437,15 +374,11 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
         int ri, rj, slot;
         const bool in = ring_cell(q, ri, rj, slot);
         const double rv0 = in ? f.R[0][g.idx(ri, rj)] : 0.0;
-        if constexpr (RES) {
-          sr[lpad(ri, rj)] = srn[lpad(ri, rj)] = rv0;  // 0 outside the domain, in both frames, for good
-          ring[slot] = 0.0;                            // s_{-1}
-        } else {
-          ring[slot] = rv0;
-        }
+        sr[lpad(ri, rj)] = srn[lpad(ri, rj)] = rv0;  // 0 outside the domain, in both frames, for good
+        ring[slot] = 0.0;                            // s_{-1}
       }
     __syncthreads();
-    stencil(f.R[0], f.W[0], 0, 1u, v);
+    stencil(0, 1u, v);
     reduce(v, 4, rows0);
     ok = sync_grid();
   }
@@ -489,8 +422,8 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     sh.lo = max(max(sc_log2(s[0]), sc_log2(s[1])), sc_log2(s[2])) + kFxMargin - kFxTop;
   };
   int cur = 0;
-  double my_w = 0.0;  // RES: w_i of this thread's first ring cell
-  if (RES && ok && sh.stop == 0 && my_in && !tag_wait(mailbox(0, tile) + my_slot, 1u, my_w, a.bar.budget, a.bar.err))
+  double my_w = 0.0;  // w_i of this thread's first ring cell
+  if (ok && sh.stop == 0 && my_in && !tag_wait(mailbox(0, tile) + my_slot, 1u, my_w, a.bar.budget, a.bar.err))
     sh.fail = 1;  // seen behind the next block barrier
   Scalar sums[3] = {};   // the last reduction's (communication warp)
   long long digit = 0;   // and this lane's digit sum of it
@@ -503,140 +436,73 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     // every block takes the same branch: the overflow count is the grid's, and the test hook
     // depends on the reduction index only
     const bool forced = f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0;
-    if constexpr (RES) {
-      // the frame that received r_i becomes the current one
-      if (defer) {
-        double* const q = sr;
-        sr = srn;
-        srn = q;
-      }
+    // the frame that received r_i becomes the current one
+    if (defer) {
+      double* const q = sr;
+      sr = srn;
+      srn = q;
     }
     v[0] = v[1] = v[2] = 0.0;
-    double* __restrict__ rn_ = f.R[nxt];
     if (comm) {
       if (rest && lane == 0) scalars_rest(sums, it);
     } else {
-      const double* __restrict__ rc_ = f.R[cur];
-      const double* __restrict__ wc_ = f.W[cur];
-      const double* __restrict__ sc_ = f.S[cur];
-      double* __restrict__ sn_ = f.S[nxt];
-      double pf_r = 0.0, pf_w = 0.0, pf_s = 0.0;
-      if constexpr (!RES) {
-        // this thread's first ring cell: the neighbours' iteration-i values, published before the
-        // last reduction, are loaded now so the L2 round trip overlaps step 1
-        if (my_in) {
-          const size_t k = g.idx(my_ri, my_rj);
-          pf_r = rc_[k];
-          pf_w = wc_[k];
-          pf_s = sc_[k];
-        }
-      }
-      // step 1: own cells (RES: in the tile; otherwise two rows of this thread at a time with
-      // their loads in flight)
-      if constexpr (RES) {
-        if (defer) {
+      // step 1: own cells
+      if (defer) {
 #pragma unroll 2
-          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
-            const double sk = sw[l] + be * ss[l];
-            ss[l] = sk;
-            srn[lp] = sr[lp] - al * sk;
-          }
-        } else {
-          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
-            const double sk = sw[l] + be * ss[l], pk = sr[lp] + be * sp[l];
-            ss[l] = sk;
-            sp[l] = pk;
-            sr[lp] -= al * sk;
-          }
+        for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+          const double sk = sw[l] + be * ss[l];
+          ss[l] = sk;
+          srn[lp] = sr[lp] - al * sk;
         }
       } else {
-        for (int q = 0; q < nq; q += 2) {
-          const bool two = q + 1 < nq;
-          const size_t ka = k0 + q * kstep, kb = two ? ka + kstep : ka;
-          const double r0 = rc_[ka], w0 = wc_[ka], s0 = sc_[ka];
-          const double r1 = rc_[kb], w1 = wc_[kb], s1 = sc_[kb];
-          const double ska = w0 + be * s0;
-          sn_[ka] = ska;
-          rn_[ka] = r0 - al * ska;
-          if (two) {
-            const double skb = w1 + be * s1;
-            sn_[kb] = skb;
-            rn_[kb] = r1 - al * skb;
-          }
+        for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+          const double sk = sw[l] + be * ss[l], pk = sr[lp] + be * sp[l];
+          ss[l] = sk;
+          sp[l] = pk;
+          sr[lp] -= al * sk;
         }
       }
-      // ring cells: r_{i+1} from the neighbours' iteration-i vectors; RES: w from the mailbox, r
-      // and s kept here (cells outside the domain stay 0)
-      if constexpr (RES) {
-        const ulonglong2* const box = mailbox(cur, tile);
-        auto ring_step = [&](int slot, int lp, double wv) {
-          const double sk = wv + be * ring[slot];
-          ring[slot] = sk;
-          srn[lp] = sr[lp] - al * sk;
-        };
-        if (my_in) ring_step(my_slot, my_lp, my_w);
-        for (int q = t + NT; q < nring; q += NT) {
-          int ri, rj, slot;
-          double wv = 0.0;
-          if (!ring_cell(q, ri, rj, slot)) continue;
-          if (!tag_wait(box + slot, tag, wv, a.bar.budget, a.bar.err)) sh.fail = 1;
-          ring_step(slot, lpad(ri, rj), wv);
-        }
-      } else {
-        if (my_ring) ring[my_slot] = my_in ? pf_r - al * (pf_w + be * pf_s) : 0.0;
-        for (int q = t + NT; q < nring; q += NT) {
-          int ri, rj, slot;
-          double rv = 0.0;
-          if (ring_cell(q, ri, rj, slot)) {
-            const size_t k = g.idx(ri, rj);
-            rv = rc_[k] - al * (wc_[k] + be * sc_[k]);
-          }
-          ring[slot] = rv;
-        }
+      // ring cells: r_{i+1} from the neighbours' w_i in the mailbox, r and s kept here (cells outside
+      // the domain stay 0)
+      const ulonglong2* const box = mailbox(cur, tile);
+      auto ring_step = [&](int slot, int lp, double wv) {
+        const double sk = wv + be * ring[slot];
+        ring[slot] = sk;
+        srn[lp] = sr[lp] - al * sk;
+      };
+      if (my_in) ring_step(my_slot, my_lp, my_w);
+      for (int q = t + NT; q < nring; q += NT) {
+        int ri, rj, slot;
+        double wv = 0.0;
+        if (!ring_cell(q, ri, rj, slot)) continue;
+        if (!tag_wait(box + slot, tag, wv, a.bar.budget, a.bar.err)) sh.fail = 1;
+        ring_step(slot, lpad(ri, rj), wv);
       }
     }
     __syncthreads();
     if (sh.stop != 0 || sh.fail) break;
     const int fx_lo = sh.lo;
     if (!comm) {
-      stencil(rn_, f.W[nxt], nxt, tag + 1u, v);
+      stencil(nxt, tag + 1u, v);
       fx_block_digits<NT>(v, fx_lo, sh.fx);
       digits_ready<NT>(false);
-      if constexpr (RES) {
-        // the neighbours' w_{i+1} arrive about when their digits do: a first look now, its answer
-        // used after the update
-        ulonglong2* const box = mailbox(nxt, tile) + my_slot;
-        bool here = true;
-        if (my_in) here = tag_get(box, tag + 1u, my_w);
-        // read by no other block and by nothing before the end
-        if (defer) {
+      // the neighbours' w_{i+1} arrive about when their digits do: a first look now, its answer
+      // used after the update
+      ulonglong2* const box = mailbox(nxt, tile) + my_slot;
+      bool here = true;
+      if (my_in) here = tag_get(box, tag + 1u, my_w);
+      // read by no other block and by nothing before the end
+      if (defer) {
 #pragma unroll 2
-          for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
-            const double pk = sr[lp] + be * sp[l];
-            sp[l] = pk;
-            sx[l] += al * pk;
-          }
-        } else {
-          for (int q = 0, l = t; q < nq; ++q, l += NT) sx[l] += al * sp[l];
+        for (int q = 0, l = t, lp = lp0; q < nq; ++q, l += NT, lp += lpstep) {
+          const double pk = sr[lp] + be * sp[l];
+          sp[l] = pk;
+          sx[l] += al * pk;
         }
-        if (!here && !tag_wait(box, tag + 1u, my_w, a.bar.budget, a.bar.err)) sh.fail = 1;
       } else {
-        const double* const rc_ = f.R[cur];
-        for (int q = 0; q < nq; q += 2) {
-          const size_t ka = k0 + q * kstep;
-          const bool two = q + 1 < nq;
-          const size_t kb = two ? ka + kstep : ka;
-          const double r0 = rc_[ka], p0 = p[ka], x0 = xs[ka], r1 = rc_[kb], p1 = p[kb], x1 = xs[kb];
-          const double pka = r0 + be * p0;
-          p[ka] = pka;
-          xs[ka] = x0 + al * pka;
-          if (two) {
-            const double pkb = r1 + be * p1;
-            p[kb] = pkb;
-            xs[kb] = x1 + al * pkb;
-          }
-        }
+        for (int q = 0, l = t; q < nq; ++q, l += NT) sx[l] += al * sp[l];
       }
+      if (!here && !tag_wait(box, tag + 1u, my_w, a.bar.budget, a.bar.err)) sh.fail = 1;
     } else {
       // The communication warp: arrive, wait, form the scalars.  Its code between the wait and the
       // barrier is on every block's critical path and runs once per iteration, with cold
@@ -650,8 +516,8 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
       for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
           digits_ready<NT>(true);
-          fx_arrive<NT, !RES>(f.fxacc, red & 1, tile == a.bar.absent, sh.fx);
-          got = fx_wait<!RES>(f.fxacc, red & 1, nb, a.bar.budget, a.bar.err, last, digit);
+          fx_arrive<NT, false>(f.fxacc, red & 1, tile == a.bar.absent, sh.fx);
+          got = fx_wait<false>(f.fxacc, red & 1, nb, a.bar.budget, a.bar.err, last, digit);
         }
         fx_sums(digit, fx_lo, sums, &over);
         if (lane == 0) {
@@ -708,7 +574,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   const bool none = ok && sh.bb == 0.0;
   for (int q = 0; q < nq; ++q) {
     const size_t k = k0 + q * kstep;
-    a.x[k] = none ? 0.0 : a.isd[k] * (RES ? sx[t + q * NT] : xs[k]);
+    a.x[k] = none ? 0.0 : a.isd[k] * sx[t + q * NT];
   }
   if (tile == 0 && t == 0) {
     const bool conv = ok && sh.stop == 1;
@@ -724,14 +590,9 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
 // __grid_constant__: the body takes the parameter by reference without a local copy.  MINB:
 // blocks per SM that must fit.
 template <int NT, int MINB>
-__global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f1(const __grid_constant__ FusedSolve f) {
-  __shared__ FusedShared<NT> sh;
-  fused_body<false, NT>(f, blockIdx.x, sh);
-}
-template <int NT, int MINB>
 __global__ void __launch_bounds__(NT + 32, MINB) k_pcg_poisson_f2(const __grid_constant__ FusedSolve f) {
   __shared__ FusedShared<NT> sh;
-  fused_body<true, NT>(f, blockIdx.x, sh);
+  fused_body<NT>(f, blockIdx.x, sh);
 }
 
 // Many cases in one cooperative launch: block b serves a tile of case block_case[b], whose tiles
@@ -743,7 +604,7 @@ __global__ void __launch_bounds__(NT + 32, MINB) k_fused_batch(const FusedBatchE
   __shared__ FusedShared<NT> sh;
   __shared__ __align__(16) unsigned char s_entry[sizeof(FusedBatchEntry)];
   const FusedBatchEntry& E = stage_entry(cases, block_case, s_entry);
-  fused_body<true, NT>(E.f, (int)blockIdx.x - E.block0, sh);
+  fused_body<NT>(E.f, (int)blockIdx.x - E.block0, sh);
 }
 
 }  // namespace
@@ -760,8 +621,8 @@ int sm_count() {
 }
 
 const void* fused_kernel(bool resident, int nt, bool two) {
-  if (nt == 128) return resident ? (const void*)k_pcg_poisson_f2<128, 2> : (const void*)k_pcg_poisson_f1<128, 2>;
-  if (!resident) return nt == 256 ? (const void*)k_pcg_poisson_f1<256, 2> : (const void*)k_pcg_poisson_f1<512, 2>;
+  if (!resident) return fused_global_kernel(nt);
+  if (nt == 128) return (const void*)k_pcg_poisson_f2<128, 2>;
   if (nt == 256) return two ? (const void*)k_pcg_poisson_f2<256, 2> : (const void*)k_pcg_poisson_f2<256, 1>;
   return two ? (const void*)k_pcg_poisson_f2<512, 2> : (const void*)k_pcg_poisson_f2<512, 1>;
 }
@@ -800,7 +661,7 @@ int fused_blocks() {
   const void* kern = fused_kernel(false, 512, true);
   int per = 0;
   allow_most_smem(kern);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 512 + 32, kFusedSmemMax);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 512, kFusedSmemMax);
   per = per > 2 ? 2 : (per < 1 ? 1 : per);
   return sm_count() * per;
 }
@@ -889,7 +750,7 @@ cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   }
   cudaMemsetAsync(f.a.bar.count, 0, sizeof(unsigned int) * kBarWords, st);
   void* params[] = {&f};
-  return cudaLaunchCooperativeKernel(kernel, f.ntiles, nt + 32, params, smem, st);
+  return cudaLaunchCooperativeKernel(kernel, f.ntiles, f.resident ? nt + 32 : nt, params, smem, st);
 }
 
 }  // namespace ccm
