@@ -1090,18 +1090,26 @@ ccm_status ccm_set_geometry(ccm_case c, const ccm_geometry* geo) {
       return fail(CCM_E_INVALID, "the body must stay two cells away from every box side");
   }
   cudaStream_t st = c->st;
-  CUDA_TRY(launch_capacities(*geo, g, c->caps.a, st));
-  // A length of a uniform grid is a difference of two abscissas x0 + i h, each rounded: the coefficients
-  // of uncut rows are off the constants by up to |x| / h units of rounding, and with a fixed tolerance
-  // most rows of a grid whose spacing is no dyadic fraction took the kernels' path for cut ones (8 FP64
-  // cases of 128..512 cells a side, advanced together: 15.5 -> 14.1 ms a step).  Mixed cases keep the
-  // fixed one: their FP32 coefficients tell (pcg_band.cu), and FP64 residuals are rare.
-  const double far_x = std::max(std::fabs(g.x0), std::fabs(g.x0 + g.nx * g.hx)) / g.hx;
-  const double far_y = std::max(std::fabs(g.y0), std::fabs(g.y0 + g.ny * g.hy)) / g.hy;
-  const bool plain = c->cfg.precision != CCM_MIXED && !g.xf && !g.yf;
-  const double uncut = 1e-14 + (plain ? 2.0 * 2.2e-16 * (far_x + far_y) : 0.0);
-  launch_derive(g, c->bc, c->ph, c->cfg.literal_offdiag, c->cfg.pressure_update, uncut, c->caps, c->co, st);
-  launch_scaling(g, uncut, c->co, st);
+  // A length of a uniform grid is a difference of two abscissas x0 + i h, each rounded: what an uncut cell
+  // measures is off h by up to three units of rounding of the largest |x|, and on a grid whose spacing is no
+  // dyadic fraction most rows then have coefficients of their own, which the kernels read (1000x500 FP64:
+  // 15.7 us per iteration instead of 11.1).  Such lengths and areas are the grid's own from the start, in the
+  // capacities themselves, so that every operator and every form of a row has the same.  (With the constants
+  // in the solver's uncut rows only, solutions met the tolerance for another operator than the projection's:
+  // 701x333 at x0 = 100, tolerance 1e-11: residual 2e-9.)  A length that a body cuts by less than the rounding
+  // of the abscissas counts as uncut; where that rounding exceeds 1e-9 of the spacing, none does.  Mixed cases
+  // keep the lengths as they come: their FP32 coefficients tell uncut rows (pcg_band.cu), and FP64 residuals
+  // are rare.
+  auto rounding = [](double x0, double h, int n) {
+    const double far = std::max(std::fabs(x0 - 3.0 * h), std::fabs(x0 + (n + 3) * h)) / h;
+    const double r = 3.0 * 2.2e-16 * far;
+    return r <= 1e-9 ? r : -1.0;
+  };
+  Snap snap{rounding(g.x0, g.hx, g.nx), rounding(g.y0, g.hy, g.ny)};
+  if (c->cfg.precision == CCM_MIXED || g.xf || g.yf || snap.x < 0.0 || snap.y < 0.0) snap = Snap{-1.0, -1.0};
+  CUDA_TRY(launch_capacities(*geo, g, snap, c->caps.a, st));
+  launch_derive(g, c->bc, c->ph, c->cfg.literal_offdiag, c->cfg.pressure_update, c->caps, c->co, st);
+  launch_scaling(g, c->co, st);
   // lifting of the box data through the viscous operator: visc(S(0, D))
   CUDA_TRY(cudaMemsetAsync(c->t0, 0, g.count() * sizeof(double), st));
   CUDA_TRY(cudaMemsetAsync(c->t1, 0, g.count() * sizeof(double), st));

@@ -262,7 +262,7 @@ struct MixedBatchEntry {
   MixedSolve a;
   int block0, nblocks;
 };
-void launch_scaling(const Geom& g, double uncut, const CoefPtrs& o, cudaStream_t st);
+void launch_scaling(const Geom& g, const CoefPtrs& o, cudaStream_t st);
 
 // One case of a batched Poisson solve and the contiguous range of blocks that serves it.
 template <class T>
@@ -369,12 +369,17 @@ void set_last_error(const char* msg);
 inline void set_last_error(const std::string& msg) { set_last_error(msg.c_str()); }
 
 // geometry.cu
-cudaError_t launch_capacities(const ccm_geometry& geo, const Geom& g, double* const* caps_dev, cudaStream_t st);
+// How far, relatively, a length along an axis may be from the uniform grid's spacing and still be taken
+// for it (negative: never)
+struct Snap {
+  double x, y;
+};
+cudaError_t launch_capacities(const ccm_geometry& geo, const Geom& g, const Snap& snap, double* const* caps_dev,
+                              cudaStream_t st);
 
 // operators.cu
-// uncut: how far, relatively, a full face's coefficient may be from the uniform grid's constant
-void launch_derive(const Geom& g, const Bc& bc, const Phys& ph, int literal, int pupdate, double uncut,
-                   const CapPtrs& cp, const CoefPtrs& o, cudaStream_t st);
+void launch_derive(const Geom& g, const Bc& bc, const Phys& ph, int literal, int pupdate, const CapPtrs& cp,
+                   const CoefPtrs& o, cudaStream_t st);
 void launch_fill_bc(const Geom& g, const Bc& bc, double* u, double* v, double scale, cudaStream_t st);
 // periodic sides: the cells beyond them take their images' values (no-op otherwise)
 void launch_wrap_cells(const Geom& g, double* p, cudaStream_t st);

@@ -14,7 +14,7 @@
 // neighbours it needs for W, so the kernel has no inter-thread dependence.
 #include <math.h>
 
-#include "ccm_internal.cuh"
+#include "ccm_host.h"
 
 namespace ccm {
 
@@ -202,7 +202,7 @@ __device__ double chord(const Piece& p, bool xaxis, double s) {
 // One cell per thread, the three grids side by side: an airfoil's crossings are bisections of some
 // fifty dependent FP64 steps in a few threads, and one grid after the other waited for them three
 // times (512x256 NACA set-up: 3.2 -> 2.0 ms).
-__global__ void k_capacities(Body b, Geom g, double* const* caps) {
+__global__ void k_capacities(Body b, Geom g, Snap snap, double* const* caps) {
   const int grid = blockIdx.z;
   const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - 1;
   const int j = (int)blockIdx.y - 1;
@@ -220,6 +220,10 @@ __global__ void k_capacities(Body b, Geom g, double* const* caps) {
   }
   for (int s = 0; s < cw.np; ++s) wx += side_area(cw.pc[s], true, cw.X - cw.xl, true);
   for (int s = 0; s < cs.np; ++s) wy += side_area(cs.pc[s], false, cs.Y - cs.yb, true);
+  // lengths and areas of uncut cells, off the grid's by the rounding of the abscissas alone
+  if (fabs(c.aleft - g.hy) <= snap.y * g.hy) c.aleft = g.hy;
+  if (fabs(c.abot - g.hx) <= snap.x * g.hx) c.abot = g.hx;
+  if (fabs(c.V - g.hx * g.hy) <= (snap.x + snap.y) * (g.hx * g.hy)) c.V = g.hx * g.hy;
   const size_t k = g.idx(i, j);
   caps[cap_slot(grid, CK_V)][k] = c.V;
   caps[cap_slot(grid, CK_X)][k] = c.X;
@@ -233,7 +237,8 @@ __global__ void k_capacities(Body b, Geom g, double* const* caps) {
 }
 
 // Host launcher: fills the 27 capacity arrays.
-cudaError_t launch_capacities(const ccm_geometry& geo, const Geom& g, double* const* caps_dev, cudaStream_t st) {
+cudaError_t launch_capacities(const ccm_geometry& geo, const Geom& g, const Snap& snap, double* const* caps_dev,
+                              cudaStream_t st) {
   Body b{};
   b.kind = geo.kind;
   b.cx = geo.cx; b.cy = geo.cy; b.r = geo.r; b.r2 = geo.r * geo.r;
@@ -245,7 +250,7 @@ cudaError_t launch_capacities(const ccm_geometry& geo, const Geom& g, double* co
   b.a4 = geo.closed_te ? -0.1036 : -0.1015;
   b.pnx = geo.hp_nx; b.pny = geo.hp_ny; b.poff = geo.hp_off;
   dim3 blk(128, 1), grd((g.nx + 3 + 127) / 128, g.ny + 3, 3);
-  k_capacities<<<grd, blk, 0, st>>>(b, g, caps_dev);
+  k_capacities<<<grd, blk, 0, st>>>(b, g, snap, caps_dev);
   return cudaGetLastError();
 }
 

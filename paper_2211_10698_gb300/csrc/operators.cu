@@ -62,7 +62,7 @@ __global__ void k_derive1(Geom g, Bc bc, Phys ph, int literal, CapPtrs cp, CoefP
   }
 }
 
-__global__ void k_derive2(Geom g, Phys ph, int pupdate, double e, CapPtrs cp, CoefPtrs o) {
+__global__ void k_derive2(Geom g, Phys ph, int pupdate, CapPtrs cp, CoefPtrs o) {
   PAD_IJ(g)
   const bool dom = i >= 0 && i < g.nx && j >= 0 && j < g.ny;
   double s = 0.0;
@@ -80,10 +80,10 @@ __global__ void k_derive2(Geom g, Phys ph, int pupdate, double e, CapPtrs cp, Co
   o.cv32[k] = (float)o.cv[k];
   o.invdk32[k] = (float)o.invdk[k];
   o.diagk32[k] = (float)o.diagk[k];
-  // row kind for the PCG: uncut rows (all four faces full, to e) use the uniform-grid constants
+  // row kind for the PCG: uncut rows (all four faces full) use the uniform-grid constants
   int8_t kind = 0;
   if (a) {
-    const double cx = g.hy / g.hx, cy = g.hx / g.hy;
+    const double cx = g.hy / g.hx, cy = g.hx / g.hy, e = 1e-14;
     const bool full = fabs(o.cu[k] - cx) <= e * cx && fabs(o.cu[k + 1] - cx) <= e * cx &&
                       fabs(o.cv[k] - cy) <= e * cy && fabs(o.cv[k + g.pitch] - cy) <= e * cy;
     kind = full ? 1 : 2;
@@ -622,10 +622,10 @@ void launch_residual64(const Coefs& c, const Geom& g, const double* x, const dou
 void launch_add_correction(const Geom& g, const int8_t* act, double* x, const float* d, cudaStream_t st) {
   k_add_correction<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, act, x, d);
 }
-void launch_derive(const Geom& g, const Bc& bc, const Phys& ph, int literal, int pupdate, double uncut,
-                   const CapPtrs& cp, const CoefPtrs& o, cudaStream_t st) {
+void launch_derive(const Geom& g, const Bc& bc, const Phys& ph, int literal, int pupdate, const CapPtrs& cp,
+                   const CoefPtrs& o, cudaStream_t st) {
   k_derive1<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, bc, ph, literal, cp, o);
-  k_derive2<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, ph, pupdate, uncut, cp, o);
+  k_derive2<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, ph, pupdate, cp, o);
 }
 void launch_fill_bc(const Geom& g, const Bc& bc, double* u, double* v, double scale, cudaStream_t st) {
   k_fill_bc<<<pad_grid(g, kBlk), kBlk, 0, st>>>(g, bc, u, v, scale);

@@ -27,7 +27,7 @@ namespace {
 // d is the diagonal of K on active cells, 1 on inactive cells (identity rows) and 0 outside
 // the domain, where every iterate is zero; 1/sqrt(d) is taken as 0 there so that faces to
 // ghost cells get a zero scaled coefficient.
-__global__ void k_scaling(Geom g, double uncut, CoefPtrs o) {
+__global__ void k_scaling(Geom g, CoefPtrs o) {
   const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - 1;
   const int j = (int)(blockIdx.y * blockDim.y + threadIdx.y) - 1;
   if (i > g.nx + 1 || j > g.ny + 1) return;
@@ -54,7 +54,7 @@ __global__ void k_scaling(Geom g, double uncut, CoefPtrs o) {
     if (o.kind[k] == 1) {
       // uncut row; the scaled row is the constant stencil when every in-domain neighbour has
       // the uncut diagonal too (ghost neighbours hold zero in every iterate)
-      const double cx = g.hy / g.hx, cy = g.hx / g.hy, dreg = 2.0 * (cx + cy), e = uncut * dreg;
+      const double cx = g.hy / g.hx, cy = g.hx / g.hy, dreg = 2.0 * (cx + cy), e = 1e-14 * dreg;
       bool uni = true;
       if (i > 0) uni = uni && fabs(o.diagk[k - 1] - dreg) <= e;
       if (i < g.nx - 1) uni = uni && fabs(o.diagk[k + 1] - dreg) <= e;
@@ -77,10 +77,10 @@ __global__ void k_scaling(Geom g, double uncut, CoefPtrs o) {
 
 }  // namespace
 
-void launch_scaling(const Geom& g, double uncut, const CoefPtrs& o, cudaStream_t st) {
+void launch_scaling(const Geom& g, const CoefPtrs& o, cudaStream_t st) {
   const dim3 b(32, 8);
   const dim3 grid((g.nx + 3 + b.x - 1) / b.x, (g.ny + 3 + b.y - 1) / b.y);
-  k_scaling<<<grid, b, 0, st>>>(g, uncut, o);
+  k_scaling<<<grid, b, 0, st>>>(g, o);
 }
 
 }  // namespace ccm
