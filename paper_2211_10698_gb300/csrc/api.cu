@@ -320,15 +320,17 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
   if (c->cfg.precond == CCM_JACOBI && !c->g.px && !c->g.py) {
     // Jacobi-PCG as CG on the symmetrically scaled system with one grid barrier per iteration
     // (tiles that recompute their ring).  A singular system takes the same iteration: with a
-    // zero-mean right-hand side its residuals stay orthogonal to the null space (the constants),
-    // so alpha, beta and r are those of the iteration that projects every preconditioned residual,
-    // and the iterates differ from its by a constant, which the last projection removes.
+    // zero-mean right-hand side its residuals stay orthogonal to the null space (the constants;
+    // the kernels take out what rounding adds), so alpha, beta and r are those of the iteration
+    // that projects every preconditioned residual, and the iterates differ from its by a constant,
+    // which the last projection removes.
     if (c->zero_mean) {
       CUDA_TRY(project_zero_mean(c->g, c->co.act, x, c->partials, c->n_act, c->st));
       CUDA_TRY(project_zero_mean(c->g, c->co.act, b, c->partials, c->n_act, c->st));
     }
     FusedSolve f = fused_solve_of(c, x, b);
     f.fx_fallback_every = c->fx_fallback_every;
+    f.zero_mean = c->zero_mean;
     f.a.partials = c->partials;
     f.a.bar = case_barrier(c);
     f.a.out = PcgOut{&c->ds->iters_p, &c->ds->rr_p, &c->ds->bb_p, &c->ds->conv_p, &c->ds->total_p, &c->ds->nconv};

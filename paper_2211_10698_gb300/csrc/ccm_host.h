@@ -127,6 +127,7 @@ struct FusedSolve {
   ScaledSolve a;
   unsigned long long* fxacc;  // kFxAccWords words (cleared by the kernel itself)
   int fx_fallback_every;      // tests only: every k-th reduction takes the FP64 fallback (0: on overflow only)
+  int zero_mean;              // singular system: the residual's null component is taken out now and then
   double* R[2];               // resident tiles use R[0] only
   double* W[2];
   double* S[2];
@@ -142,7 +143,8 @@ struct FusedSolve {
   int defer;                // (resident) a second r frame, so that p waits for the barrier as x does
 };
 cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st);
-const void* fused_global_kernel(int nt);  // tiles in global memory, nt threads per block (pcg_fused_global.cu)
+// tiles in global memory, nt threads per block (pcg_fused_global.cu)
+const void* fused_global_kernel(int nt, bool zero_mean);
 // One case of a batched launch of resident tiles: its first block (one block per tile).
 struct FusedBatchEntry {
   FusedSolve f;

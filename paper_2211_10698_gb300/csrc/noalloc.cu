@@ -127,6 +127,7 @@ extern "C" ccm_status ccm_solve_pressure_noalloc(ccm_case c, const double* rhs_d
   f.mail = S->mail;
   f.mail_slots = 2 * kMaxElems;
   f.resident = 1;
+  f.zero_mean = v.zero_mean;
   e = cudaSuccess;
   if (v.zero_mean) {
     e = project_zero_mean(v.g, v.act, phi_dev, S->partials, v.n_act, st);

@@ -67,6 +67,7 @@ struct FusedShared {
   double bsum[8];
   double gsum[8];
   double alpha, beta, rr, bb;
+  double nn;  // singular systems: squared norm of the null vector, sum of d over the active cells
   int stop, lo, redo, fail;
   int scan[NT / 32 + 1];
   FxShared<NT> fx;
@@ -380,7 +381,20 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     __syncthreads();
     stencil(0, 1u, v);
     reduce(v, 4, rows0);
+    if (f.zero_mean) {
+      double n[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int q = 0; q < nq; ++q) {
+        const size_t k = k0 + q * kstep;
+        if (kinds[k] != 0) n[0] += sd[k] * sd[k];
+      }
+      reduce(n, 1, rows1);
+    }
     ok = sync_grid();
+    if (ok && f.zero_mean) {
+      double n[1];
+      grid_sum<1>(rows1, nb, n, sh.gsum);
+      if (t == 0) sh.nn = n[0];
+    }
   }
   // The communication warp's state: the recurrence, and its lanes' words after their last use
   // (of the buffer next in turn and of the other).
@@ -435,7 +449,8 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     const double al = sh.alpha, be = sh.beta;
     // every block takes the same branch: the overflow count is the grid's, and the test hook
     // depends on the reduction index only
-    const bool forced = f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0;
+    const bool forced = (f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0) ||
+                        (f.zero_mean != 0 && red % kZeroMeanEvery == 1);
     // the frame that received r_i becomes the current one
     if (defer) {
       double* const q = sr;
@@ -544,10 +559,34 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
       // a value outside the window (every block sees the same count): this reduction again in
       // FP64 through the partial rows and the counter barrier
       double* const rows = (it & 1) ? rows0 : rows1;
-      reduce(v, 3, rows);
-      if (!sync_grid()) { ok = false; break; }
-      double d[3];
-      grid_sum<3>(rows, nb, d, sh.gsum);
+      double d[4];
+      if (f.zero_mean) {
+        // ... with (n, r), n = D^1/2 1, and r -= n (n, r) / (n, n) on the tile and its ring
+        v[3] = 0.0;
+        for (int q = 0, lp = lp0; q < nq; ++q, lp += lpstep) v[3] += sd[k0 + q * kstep] * srn[lp];
+        reduce(v, 4, rows);
+        if (!sync_grid()) { ok = false; break; }
+        grid_sum<4>(rows, nb, d, sh.gsum);
+        const double c = d[3] / sh.nn;
+        for (int q = 0, lp = lp0; q < nq; ++q, lp += lpstep) {
+          const size_t k = k0 + q * kstep;
+          if (kinds[k] != 0) srn[lp] = fma(-c, sd[k], srn[lp]);
+        }
+        if (!comm)
+          for (int q = t; q < nring; q += NT) {
+            int ri, rj, slot;
+            if (!ring_cell(q, ri, rj, slot)) continue;
+            const size_t k = g.idx(ri, rj);
+            if (kinds[k] != 0) srn[lpad(ri, rj)] = fma(-c, sd[k], srn[lpad(ri, rj)]);
+          }
+        d[0] -= c * d[3];
+      } else {
+        reduce(v, 3, rows);
+        if (!sync_grid()) { ok = false; break; }
+        double d3[3];
+        grid_sum<3>(rows, nb, d3, sh.gsum);
+        d[0] = d3[0]; d[1] = d3[1]; d[2] = d3[2];
+      }
       if (comm) {
         if (isfinite(d[0]) && isfinite(d[1]) && isfinite(d[2])) {
 #pragma unroll
@@ -620,8 +659,7 @@ int sm_count() {
   return sms;
 }
 
-const void* fused_kernel(bool resident, int nt, bool two) {
-  if (!resident) return fused_global_kernel(nt);
+const void* fused_kernel(int nt, bool two) {
   if (nt == 128) return (const void*)k_pcg_poisson_f2<128, 2>;
   if (nt == 256) return two ? (const void*)k_pcg_poisson_f2<256, 2> : (const void*)k_pcg_poisson_f2<256, 1>;
   return two ? (const void*)k_pcg_poisson_f2<512, 2> : (const void*)k_pcg_poisson_f2<512, 1>;
@@ -633,7 +671,7 @@ const void* fused_kernel(bool resident, int nt, bool two) {
 size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
   const int sms = sm_count(), nt = fused_threads(TX, TY, ntiles, sms);
   if (ntiles < 1 || ntiles > 2 * sms || TX * TY > kFusedRows * nt) return 0;
-  const void* kern = fused_kernel(true, nt, ntiles > sms);
+  const void* kern = fused_kernel(nt, ntiles > sms);
   const size_t room = allow_most_smem(kern);
   for (int k = 7; k >= 0; --k) {
     const bool dc = (k & 4) != 0, df = (k & 2) != 0, lc = (k & 1) != 0;
@@ -658,7 +696,7 @@ size_t resident_shape(int TX, int TY, int ntiles, FusedSolve* f) {
 }  // namespace
 
 int fused_blocks() {
-  const void* kern = fused_kernel(false, 512, true);
+  const void* kern = fused_global_kernel(512, true);
   int per = 0;
   allow_most_smem(kern);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 512, kFusedSmemMax);
@@ -731,7 +769,7 @@ cudaError_t run_poisson_fused(FusedSolve f, cudaStream_t st) {
   }
   if (f.ntiles < 1) return cudaErrorInvalidConfiguration;
   const int nt = fused_threads(f.TX, f.TY, f.ntiles, sms);
-  const void* kernel = fused_kernel(f.resident != 0, nt, f.ntiles > sms);
+  const void* kernel = f.resident ? fused_kernel(nt, f.ntiles > sms) : fused_global_kernel(nt, f.zero_mean != 0);
   size_t smem = 0;
   f.wx = std::min(f.TX, f.a.g.nx);
   if (f.resident) {

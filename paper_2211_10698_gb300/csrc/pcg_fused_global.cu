@@ -33,6 +33,7 @@ struct GlobalShared {
   double bsum[8];
   double gsum[8];
   double alpha, beta, rr, bb, thr;  // thr: tol^2 ||b||^2
+  double nn;                        // singular systems: sum of d over the active cells
   Scalar sums[3], den, igamma[2];   // the last reduction's sums; the recurrence, 1 / gamma by parity
   unsigned long long last[2][32];   // words of either buffer after their last use, by lane
   int stop, lo, over, got;
@@ -40,7 +41,8 @@ struct GlobalShared {
   FxShared<NT> fx;
 };
 
-template <int NT, int MINB>
+// ZM: singular system
+template <bool ZM, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_pcg_poisson_f1(const __grid_constant__ FusedSolve f) {
   __shared__ GlobalShared<NT> sh;
   // dynamic shared memory: the ring's r~ [W: TY][E: TY][S: TX][N: TX], then the list
@@ -258,7 +260,21 @@ __global__ void __launch_bounds__(NT, MINB) k_pcg_poisson_f1(const __grid_consta
     __syncthreads();
     stencil(f.R[0], f.W[0], v);
     reduce(v, 4, rows0);
+    if constexpr (ZM) {
+      double n[4] = {0.0, 0.0, 0.0, 0.0};
+      if (col)
+        for (int j = j0 + ty0; j < j1; j += RP) {
+          const size_t k = g.idx(ci, j);
+          if (kinds[k] != 0) n[0] += sd[k] * sd[k];
+        }
+      reduce(n, 1, rows1);
+    }
     ok = grid_sync(a.bar, target);
+    if constexpr (ZM) {
+      double n[1] = {0.0};
+      if (ok) grid_sum<1>(rows1, nb, n, sh.gsum);
+      if (t == 0) sh.nn = n[0];
+    }
   }
   if (ok) {
     double s[4];
@@ -379,14 +395,35 @@ __global__ void __launch_bounds__(NT, MINB) k_pcg_poisson_f1(const __grid_consta
     // every block takes the same branch: the overflow count is the grid's, and the test hook depends on
     // the reduction index only
     bool finite = true;
-    if (sh.over != 0 || (f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0)) {
+    if (sh.over != 0 || (f.fx_fallback_every > 0 && red % f.fx_fallback_every == 0) ||
+        (ZM && red % kZeroMeanEvery == 1)) {
       // a value outside the window: this reduction again in FP64 through the partial rows and the
       // counter barrier
       double* const rows = (it & 1) ? rows0 : rows1;
-      reduce(v, 3, rows);
-      if (!grid_sync(a.bar, target)) { ok = false; break; }
-      double d[3];
-      grid_sum<3>(rows, nb, d, sh.gsum);
+      double d[4];
+      if constexpr (ZM) {
+        // ... with (n, r), n = D^1/2 1, and r -= n (n, r) / (n, n), which the neighbours' rings read next
+        v[3] = 0.0;
+        if (col)
+          for (int j = j0 + ty0; j < j1; j += RP) v[3] += sd[g.idx(ci, j)] * rn_[g.idx(ci, j)];
+        reduce(v, 4, rows);
+        if (!grid_sync(a.bar, target)) { ok = false; break; }
+        grid_sum<4>(rows, nb, d, sh.gsum);
+        const double c = d[3] / sh.nn;
+        if (col)
+          for (int j = j0 + ty0; j < j1; j += RP) {
+            const size_t k = g.idx(ci, j);
+            if (kinds[k] != 0) rn_[k] = fma(-c, sd[k], rn_[k]);
+          }
+        if (!grid_sync(a.bar, target)) { ok = false; break; }
+        d[0] -= c * d[3];
+      } else {
+        reduce(v, 3, rows);
+        if (!grid_sync(a.bar, target)) { ok = false; break; }
+        double d3[3];
+        grid_sum<3>(rows, nb, d3, sh.gsum);
+        d[0] = d3[0]; d[1] = d3[1]; d[2] = d3[2];
+      }
       finite = isfinite(d[0]) && isfinite(d[1]) && isfinite(d[2]);
       if (t == 0) {
         if (finite) {
@@ -424,9 +461,12 @@ __global__ void __launch_bounds__(NT, MINB) k_pcg_poisson_f1(const __grid_consta
 
 }  // namespace
 
-const void* fused_global_kernel(int nt) {
-  return nt == 128 ? (const void*)k_pcg_poisson_f1<128, 2>
-                   : nt == 256 ? (const void*)k_pcg_poisson_f1<256, 2> : (const void*)k_pcg_poisson_f1<512, 2>;
+const void* fused_global_kernel(int nt, bool zero_mean) {
+  if (zero_mean)
+    return nt == 128 ? (const void*)k_pcg_poisson_f1<true, 128, 2>
+                     : nt == 256 ? (const void*)k_pcg_poisson_f1<true, 256, 2> : (const void*)k_pcg_poisson_f1<true, 512, 2>;
+  return nt == 128 ? (const void*)k_pcg_poisson_f1<false, 128, 2>
+                   : nt == 256 ? (const void*)k_pcg_poisson_f1<false, 256, 2> : (const void*)k_pcg_poisson_f1<false, 512, 2>;
 }
 
 }  // namespace ccm
