@@ -59,17 +59,27 @@ __host__ __device__ __forceinline__ Scalar sc_of_double(double x) {
   return sc_of_u128(0ULL, m, ex != 0 ? ex - 1075 : -1074, (b >> 63) != 0);
 }
 
-// Rounded to nearest (ties to even) FP64; beyond its range infinite, below it 0.
+// Rounded to nearest (ties to even) FP64, subnormals included; beyond its range infinite.
 __host__ __device__ __forceinline__ double sc_double(const Scalar& a) {
   const unsigned long long sign = a.neg ? 1ULL << 63 : 0ULL;
   if (a.m == 0) return fx_double((long long)sign);
+  int E = a.e + 63 + 1023;
+  if (E < 1) {
+    // subnormal: fewer bits are kept (a residual norm near the end of a solve with tiny right-hand side;
+    // flushed to 0 it would meet any tolerance)
+    const int shift = 12 - E;
+    if (shift > 64) return fx_double((long long)sign);
+    const unsigned long long half = 1ULL << (shift - 1);
+    const unsigned long long rest = shift == 64 ? a.m : a.m & ((half << 1) - 1);
+    unsigned long long t = shift == 64 ? 0ULL : a.m >> shift;
+    if (rest > half || (rest == half && (t & 1))) t += 1;  // (2^52 is the smallest normal number)
+    return fx_double((long long)(sign | t));
+  }
   unsigned long long t = a.m >> 11;
   const unsigned long long rem = a.m & 0x7ffULL;
-  int E = a.e + 63 + 1023;
   if (rem > 0x400ULL || (rem == 0x400ULL && (t & 1))) t += 1;
   if (t >> 53) { t >>= 1; E += 1; }
   if (E > 2046) return fx_double((long long)(sign | (0x7ffULL << 52)));
-  if (E < 1) return fx_double((long long)sign);
   return fx_double((long long)(sign | ((unsigned long long)E << 52) | (t & 0xfffffffffffffULL)));
 }
 
