@@ -277,6 +277,11 @@ ccm_status ccm_step(ccm_case c, int nsteps, ccm_step_stats* stats);
  * cluster barrier and is not affected.  CCM_E_INVALID for budget_cycles < 0 or
  * absent_block < -1. */
 ccm_status ccm_set_barrier_fault(ccm_case c, long long budget_cycles, int absent_block);
+/* The same for the words that neighbouring tiles exchange (resident FP64 tiles, mixed band tiles):
+ * block silent_block of each such launch passes every barrier but sends its neighbours nothing (-1:
+ * none, the default), so that their waits run out while the other blocks still iterate.  CCM_E_INVALID
+ * for silent_block < -1. */
+ccm_status ccm_set_mailbox_fault(ccm_case c, int silent_block);
 
 /* Test hook for the exact fixed-point dot products of the FP64 one-barrier CG (the paper has
  * no counterpart): with every = k > 0, every k-th reduction of a solve also takes the FP64

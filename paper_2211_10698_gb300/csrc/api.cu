@@ -115,7 +115,7 @@ struct ccm_case_s {
   // device-wide barriers of the case's cooperative launches: the spin budget, and the block
   // that skips its arrivals (failure-detection tests only; -1 otherwise)
   long long bar_budget = kBarrierBudget;
-  int bar_absent = -1;
+  int bar_absent = -1, bar_silent = -1;
   // tests only: every k-th fixed-point reduction of the FP64 one-barrier CG takes its FP64
   // fallback (0: only when a value leaves the window)
   int fx_fallback_every = 0;
@@ -135,6 +135,7 @@ namespace {
 Barrier case_barrier(ccm_case c) {
   Barrier b{c->bar_count, c->bar_err, c->bar_budget};
   b.absent = c->bar_absent;
+  b.silent = c->bar_silent;
   return b;
 }
 
@@ -1498,6 +1499,14 @@ ccm_status ccm_set_barrier_fault(ccm_case c, long long budget_cycles, int absent
   if (budget_cycles < 0 || absent_block < -1) return fail(CCM_E_INVALID, "budget_cycles >= 0, absent_block >= -1");
   c->bar_budget = budget_cycles > 0 ? budget_cycles : kBarrierBudget;
   c->bar_absent = absent_block;
+  return CCM_OK;
+}
+
+ccm_status ccm_set_mailbox_fault(ccm_case c, int silent_block) {
+  g_last_error.clear();
+  if (!c) return fail(CCM_E_INVALID, "null case");
+  if (silent_block < -1) return fail(CCM_E_INVALID, "silent_block >= -1");
+  c->bar_silent = silent_block;
   return CCM_OK;
 }
 

@@ -148,6 +148,7 @@ struct Barrier {
   long long budget;     // clock64 cycles a block waits before it gives up
   int absent = -1;      // failure-detection tests only: this block never arrives, so every other
                         // block's wait runs out; -1 in every normal launch
+  int silent = -1;      // likewise: this block arrives but sends its neighbours nothing
 };
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {

@@ -343,9 +343,10 @@ __device__ __forceinline__ int band_segment(const BandSolve& f, const int tile, 
   };
   const unsigned int rows_in = bits(max(0, T.h - T.j0), min(T.rows, g.ny - T.j0 + T.h));  // in the domain
   const unsigned int rows_own = bits(T.h, T.h + T.Ht);
-  const unsigned int rows_frame = rows_own & ~bits(2 * T.h, T.Ht);
+  const bool sends = tile != f.m.d.bar.silent;
+  const unsigned int rows_frame = sends ? rows_own & ~bits(2 * T.h, T.Ht) : 0u;
   const bool live = lane < T.live, own = col >= 0 && col < T.Wt;
-  const bool frame_col = col < T.hp || col + 3 >= T.Wt - T.hp;
+  const bool frame_col = sends && (col < T.hp || col + 3 >= T.Wt - T.hp);
   const bool in_col = live && T.i0 + col >= 0 && T.i0 + col < g.nx;
   const int woff = word(g, T.i0 + col, T.j0 - T.h + r0);
 

@@ -68,7 +68,10 @@ struct FusedShared {
   double gsum[8];
   double alpha, beta, rr, bb;
   double nn;  // singular systems: squared norm of the null vector, sum of d over the active cells
-  int stop, lo, redo, fail;
+  int stop, lo, redo;
+  // a wait that ran out: before the block barrier that ends step 1 (fail) and after it (late); each is read
+  // behind the barrier that follows its waits and written again only behind the next one
+  int fail, late;
   int scan[NT / 32 + 1];
   FxShared<NT> fx;
 };
@@ -145,9 +148,10 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
   auto mailbox = [&](int parity, int q) -> ulonglong2* { return f.mail + ((size_t)parity * nb + q) * nslot; };
   // w~ of a perimeter cell to the ring of every neighbour that reads it: first slots of the
   // neighbours' rows (columns) that face this tile, -1 where there is no neighbour
-  const int slotW = bx > 0 ? (tile - 1) * nslot + TY : -1, slotE = i1 < nx ? (tile + 1) * nslot : -1;
-  const int slotS = by > 0 ? (tile - f.nbx) * nslot + 2 * TY + f.wx : -1;
-  const int slotN = j1 < ny ? (tile + f.nbx) * nslot + 2 * TY : -1;
+  const bool sends = tile != a.bar.silent;
+  const int slotW = sends && bx > 0 ? (tile - 1) * nslot + TY : -1, slotE = sends && i1 < nx ? (tile + 1) * nslot : -1;
+  const int slotS = sends && by > 0 ? (tile - f.nbx) * nslot + 2 * TY + f.wx : -1;
+  const int slotN = sends && j1 < ny ? (tile + f.nbx) * nslot + 2 * TY : -1;
   const int hi_ = i1 - i0 - 1, hj_ = j1 - j0 - 1;  // last column and row
   // (ir, jr): the cell within the tile
   auto push = [&](int parity, unsigned int tag, int ir, int jr, double wk) {
@@ -214,7 +218,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
         acc += c;
       }
       sh.scan[NT / 32] = acc;
-      sh.fail = 0;
+      sh.fail = sh.late = 0;
     }
     __syncthreads();
     nlist = sh.scan[NT / 32];
@@ -517,7 +521,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
       } else {
         for (int q = 0, l = t; q < nq; ++q, l += NT) sx[l] += al * sp[l];
       }
-      if (!here && !tag_wait(box, tag + 1u, my_w, a.bar.budget, a.bar.err)) sh.fail = 1;
+      if (!here && !tag_wait(box, tag + 1u, my_w, a.bar.budget, a.bar.err)) sh.late = 1;
     } else {
       // The communication warp: arrive, wait, form the scalars.  Its code between the wait and the
       // barrier is on every block's critical path and runs once per iteration, with cold
@@ -550,11 +554,11 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
       if (rest) st = next;
       if (lane == 0) {
         sh.redo = forced || over != 0;
-        if (!got) sh.fail = 1;
+        if (!got) sh.late = 1;
       }
     }
     __syncthreads();
-    if (sh.fail) { ok = false; break; }
+    if (sh.late) { ok = false; break; }
     if (sh.redo) {
       // a value outside the window (every block sees the same count): this reduction again in
       // FP64 through the partial rows and the counter barrier
@@ -608,7 +612,7 @@ __device__ __forceinline__ void fused_body(const FusedSolve& f, const int tile, 
     it = red;
     cur = nxt;
   }
-  if (sh.fail) ok = false;
+  if (sh.fail) ok = false;  // (left behind step 1)
   // b = 0: the solution is 0, whatever the warm start was
   const bool none = ok && sh.bb == 0.0;
   for (int q = 0; q < nq; ++q) {
