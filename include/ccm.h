@@ -97,7 +97,7 @@ typedef struct {
   int autotune;               /* 1: set_geometry times candidate launch shapes of the case's
                                  one-launch Poisson solve (FP64 Jacobi: the tile plan; MIXED: the
                                  block count) on a short scratch solve and keeps the fastest,
-                                 cached per grid size for the process; 0: the built-in plan.
+                                 cached per grid size and kind of mesh for the process; 0: the built-in plan.
                                  Batched solves (ccm_batch_*) do not use it. */
   ccm_alloc_fn alloc;
   ccm_free_fn free;

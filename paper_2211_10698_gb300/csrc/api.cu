@@ -531,7 +531,7 @@ ccm_status autotune_poisson(ccm_case c) {
   const int most = mixed ? mixed_blocks() : fused_blocks();
   const int deg = c->cfg.precond == CCM_CHEBYSHEV ? c->cfg.cheb_degree : 1;
   TuneResult r{};
-  if (tune_cache_get(g.nx, g.ny, c->cfg.precision, c->cfg.precond, deg, most, &r)) {
+  if (tune_cache_get(g, c->cfg.precision, c->cfg.precond, deg, most, &r)) {
     c->tune = r;
     return CCM_OK;
   }
@@ -611,7 +611,7 @@ ccm_status autotune_poisson(ccm_case c) {
   CUDA_TRY(cudaMemcpyAsync(&bar_err, c->bar_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   if (bar_err) return fail(CCM_E_TIMEOUT, "autotune: a device-wide barrier gave up waiting");
-  if (best >= 0) tune_cache_put(g.nx, g.ny, c->cfg.precision, c->cfg.precond, deg, most, r);
+  if (best >= 0) tune_cache_put(g, c->cfg.precision, c->cfg.precond, deg, most, r);
   c->tune = r;
   return CCM_OK;
 }

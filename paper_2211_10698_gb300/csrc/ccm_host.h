@@ -182,8 +182,8 @@ struct TuneResult {
 std::vector<TilePlan> fused_plan_candidates(int nx, int ny, int blocks);
 std::vector<int> mixed_block_candidates(int blocks);
 std::vector<int> cluster_candidates(int nx, int ny);
-bool tune_cache_get(int nx, int ny, int precision, int precond, int degree, int blocks, TuneResult* r);
-void tune_cache_put(int nx, int ny, int precision, int precond, int degree, int blocks, const TuneResult& r);
+bool tune_cache_get(const Geom& g, int precision, int precond, int degree, int blocks, TuneResult* r);
+void tune_cache_put(const Geom& g, int precision, int precond, int degree, int blocks, const TuneResult& r);
 // Times launch(k) for k = 0 .. n-1 with CUDA events on st (after one untimed launch(0));
 // candidates whose launch returns cudaErrorInvalidConfiguration are skipped.  best = the
 // fastest index, ms = the times (-1 where skipped).

@@ -6,7 +6,9 @@
 // grid wants every SM busy, a small one loses more to the grid barrier across many blocks
 // than it gains from them.  The caller times each candidate on a short solve of the case's
 // own operator (a fixed number of iterations on a scratch right-hand side) and keeps the
-// fastest; results are cached per grid size and solver setting for the life of the process.
+// fastest; results are cached per grid size, kind of mesh (a stretched one has coefficients for every
+// row, so that other tiles fit and other shapes are fast) and solver setting for the life of the
+// process.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -63,23 +65,24 @@ std::vector<int> cluster_candidates(int nx, int ny) {
 
 namespace {
 
-using Key = std::tuple<int, int, int, int, int, int>;  // nx, ny, precision, precond, degree, blocks
+// nx, ny, stretched, precision, precond, degree, blocks
+using Key = std::tuple<int, int, bool, int, int, int, int>;
 std::mutex g_tune_mutex;
 std::map<Key, TuneResult> g_tune_cache;
 
 }  // namespace
 
-bool tune_cache_get(int nx, int ny, int precision, int precond, int degree, int blocks, TuneResult* r) {
+bool tune_cache_get(const Geom& g, int precision, int precond, int degree, int blocks, TuneResult* r) {
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  auto it = g_tune_cache.find(Key{nx, ny, precision, precond, degree, blocks});
+  auto it = g_tune_cache.find(Key{g.nx, g.ny, g.xf || g.yf, precision, precond, degree, blocks});
   if (it == g_tune_cache.end()) return false;
   *r = it->second;
   return true;
 }
 
-void tune_cache_put(int nx, int ny, int precision, int precond, int degree, int blocks, const TuneResult& r) {
+void tune_cache_put(const Geom& g, int precision, int precond, int degree, int blocks, const TuneResult& r) {
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  g_tune_cache[Key{nx, ny, precision, precond, degree, blocks}] = r;
+  g_tune_cache[Key{g.nx, g.ny, g.xf || g.yf, precision, precond, degree, blocks}] = r;
 }
 
 cudaError_t time_launches(int n, const std::function<cudaError_t(int)>& launch, cudaStream_t st, int* best,
