@@ -450,6 +450,8 @@ def _measure_case(torch, stream, flush, case, steps, warmup, precision=None, pre
 def _plan_dict(g, precision="fp64"):
     """The launch shape the set-up autotuner chose for the case's Poisson solve (a mixed case's
     tiles are those of the solve with one barrier per iteration)."""
+    from paper_2211_10698_gb300 import ccm
+
     tx, ty, nbx, ntiles, mb, cl, res = g.launch_plan()
     if cl:
         return dict(kind="cluster", ctas=cl)
@@ -457,6 +459,8 @@ def _plan_dict(g, precision="fp64"):
         return dict(kind="tiles, one barrier per iteration", tile=[tx, ty], tiles=ntiles, resident=bool(res))
     if tx:
         return dict(kind="tiles", tile=[tx, ty], tiles=ntiles, resident=bool(res))
+    if mb > ccm.CCM_PLAN_BAND:
+        return dict(kind="resident band tiles", tiles=mb - ccm.CCM_PLAN_BAND)
     if mb:
         return dict(kind="blocks", blocks=mb, precision=precision)
     return dict(kind="built-in", precision=precision)

@@ -17,6 +17,7 @@ import numpy as np
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libccm.so")
 
 CCM_OK, CCM_E_INVALID, CCM_E_OOM, CCM_E_CUDA, CCM_E_NOT_CONVERGED, CCM_E_NONFINITE, CCM_E_TIMEOUT, CCM_E_STATE = range(8)
+CCM_PLAN_BAND = 65536  # launch_plan()[4]: the resident band's tiles are counted from here
 STATUS_NAMES = ["CCM_OK", "CCM_E_INVALID", "CCM_E_OOM", "CCM_E_CUDA", "CCM_E_NOT_CONVERGED", "CCM_E_NONFINITE",
                 "CCM_E_TIMEOUT", "CCM_E_STATE"]
 CCM_BC_DIRICHLET, CCM_BC_OUTFLOW, CCM_BC_PERIODIC = 0, 1, 2
@@ -275,8 +276,9 @@ class Case:
         return {f: getattr(st, f) for f, _ in ccm_step_stats._fields_}
 
     def launch_plan(self):
-        """(tile width, tile height, tiles per row, tiles, mixed blocks, cluster CTAs, resident
-        tiles) of the single-case Poisson solve; zeros where the built-in shape is used."""
+        """(tile width, tile height, tiles per row, tiles, mixed blocks or CCM_PLAN_BAND + band tiles,
+        cluster CTAs, resident tiles) of the single-case Poisson solve; zeros where the built-in shape
+        is used."""
         plan = (c_int * 7)()
         _check(lib().ccm_launch_plan(self.h, plan))
         return tuple(plan)

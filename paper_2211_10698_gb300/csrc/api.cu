@@ -342,7 +342,8 @@ ccm_status solve_poisson_fp64(ccm_case c, double* x, double* b) {
       CUDA_TRY(run_poisson_cluster(cs, c->tune.cluster, c->st));
       return CCM_OK;
     }
-    const TilePlan& tp = c->tune.plan;
+    // (a singular system takes the built-in shape whatever plan is set)
+    const TilePlan tp = c->zero_mean ? TilePlan{} : c->tune.plan;
     f.TX = tp.TX; f.TY = tp.TY; f.nbx = tp.nbx; f.ntiles = tp.ntiles; f.resident = tp.resident;
     CUDA_TRY(run_poisson_fused(f, c->st));
     if (c->zero_mean) CUDA_TRY(project_zero_mean(c->g, c->co.act, x, c->partials, c->n_act, c->st));
@@ -958,7 +959,7 @@ ccm_status ccm_launch_plan(ccm_case c, int plan[7]) {
   plan[1] = tp.TY;
   plan[2] = tp.nbx;
   plan[3] = tp.ntiles;
-  plan[4] = c->tune.band > 0 ? c->tune.band : c->tune.mixed_blocks;
+  plan[4] = c->tune.band > 0 ? CCM_PLAN_BAND + c->tune.band : c->tune.mixed_blocks;
   plan[5] = c->tune.cluster;
   plan[6] = tp.resident;
   return CCM_OK;
@@ -1001,16 +1002,18 @@ ccm_status ccm_set_launch_plan(ccm_case c, const int plan[7]) {
   } else if (plan[6] != 0) {
     return fail(CCM_E_INVALID, "resident tiles need a tile plan");
   }
-  if (plan[4] < 0 || plan[4] > mixed_blocks()) return fail(CCM_E_INVALID, "mixed blocks out of range");
-  // as many blocks as the resident band has tiles: that solve, as ccm_launch_plan reports it
-  if (mixed && plan[4] > 0 && !c->zero_mean && !c->g.px && !c->g.py) {
+  if (mixed && plan[4] > CCM_PLAN_BAND && !c->zero_mean && !c->g.px && !c->g.py) {
     MixedSolve a{};
     case_mixed_solve(c, nullptr, nullptr, &a);
     BandSolve bs{};
     case_band_solve(c, a, &bs);
-    if (band_fits(&bs) && bs.ntiles == plan[4]) r.band = plan[4];
+    if (!band_fits(&bs) || bs.ntiles != plan[4] - CCM_PLAN_BAND)
+      return fail(CCM_E_INVALID, "band tiles: not as many as the case's, or they do not fit the GPU");
+    r.band = bs.ntiles;
+  } else {
+    if (plan[4] < 0 || plan[4] > mixed_blocks()) return fail(CCM_E_INVALID, "mixed blocks out of range");
+    r.mixed_blocks = plan[4];
   }
-  if (r.band == 0) r.mixed_blocks = plan[4];
   if (plan[5] != 0) {
     bool ok = false;
     for (int C : cluster_candidates(g.nx, g.ny)) ok = ok || C == plan[5];
