@@ -258,10 +258,9 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   __shared__ float wred[3][kPcgThreads / 32];
   __shared__ double dsum[8];
   __shared__ float fsum[8];
-  __shared__ double sc_sigma, sc_rr, sc_bb, sc_rr_ref, sc_racc[3];
+  __shared__ double sc_sigma, sc_rr, sc_bb, sc_rr_ref;
   __shared__ float sc_alpha, sc_beta, sc_pscale, sc_igamma, sc_ialpha, sc_gref, sc_gfresh;
-  __shared__ int sc_slot, sc_part, sc_fresh, sc_it, sc_stop, sc_nrep, sc_rep_it, sc_keep, sc_restart, sc_final,
-      sc_init;
+  __shared__ int sc_slot, sc_fresh, sc_it, sc_stop, sc_nrep, sc_rep_it, sc_keep, sc_restart, sc_final, sc_init;
   unsigned int target = 0;
   const int NB = gridDim.x;
   __shared__ __align__(16) unsigned char s_entry[sizeof(MixedBatchEntry)];
@@ -272,9 +271,6 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   const int nx = g.nx;
   const int lb = blockIdx.x - E.block0, nbc = E.nblocks;
   const CaseRange ch(g.nx * g.ny, lb, nbc);
-  // The FP64 residual of a replacement is one slot: with per-case barriers no other case waits
-  // for it (the slot code still takes it in parts when asked to).
-  const int nparts = 1;
   unsigned int* const case_bar = ctl.case_bar + (size_t)kCaseBarStride * block_case[blockIdx.x];
   // the FP32 phases work on aligned quads of the case's arrays (see QuadOpsF32)
   const Quads Q(g);
@@ -296,7 +292,6 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
 
   if (threadIdx.x == 0) {
     sc_slot = SL_FOLD;
-    sc_part = 0;
     sc_init = 1;
     sc_sigma = 0.0;
     sc_bb = 0.0;
@@ -313,9 +308,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
   // The slot after one without sums is known to every thread; after sums thread 0 decides.
   int sl = SL_FOLD, step = 1;
   for (unsigned int t = 0; ok; ++t) {
-    const int part = sc_part;
     if (sl == SL_DONE) break;  // every block of the case sees the same slot
-    const bool last_part = part == nparts - 1;
     double* prow = ctl.partials + (size_t)(3 * (t & 1)) * NB;
     if (sl == SL_FOLD) {
       if (sc_init) {
@@ -330,14 +323,11 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
         for (int u = ufirst, k0 = kfirst; u < u1; u += blockDim.x, k0 = u < u1 ? Q.k(u) : 0) quad_fold(d.x, d.isd, e, k0, isig, true);
       }
     } else if (sl == SL_RESID) {
-      // part `part` of the block's cells: r64 = D^-1/2 (b - K x) and the norms, summed over
-      // the parts in shared memory and published with the last
+      // r64 = D^-1/2 (b - K x) and the norms, in one slot: with per-case barriers no other case
+      // waits for it
       const KRow<double> K{d.cu, d.cv, d.dk, d.kind, d.creg_x, d.creg_y, d.dreg, (size_t)g.pitch};
-      const int len = ch.t1 - ch.t0;
-      const int a0 = ch.t0 + (int)((long long)len * part / nparts);
-      const int a1 = ch.t0 + (int)((long long)len * (part + 1) / nparts);
       double v[3] = {0.0, 0.0, 0.0};
-      for (CellWalk cw(a0 + threadIdx.x, blockDim.x, a1, nx); cw.ok(); cw.next()) {
+      for (CellWalk cw(ch.t0 + threadIdx.x, blockDim.x, ch.t1, nx); cw.ok(); cw.next()) {
         const size_t k = g.idx(cw.i, cw.j);
         const double bk = d.b[k];
         const double rk = bk - K(d.x, k);
@@ -348,10 +338,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
         v[2] += bk * bk;
       }
       block_sum_warps<3>(v, red, dsum);
-      if (threadIdx.x == 0) {
-        for (int q = 0; q < 3; ++q) sc_racc[q] = part == 0 ? dsum[q] : sc_racc[q] + dsum[q];
-        if (last_part) publish(prow, NB, sc_racc, 3);
-      }
+      publish(prow, NB, dsum, 3);
     } else if (sl == SL_FRESH) {
       const double sig = sc_sigma;
       if (cheb == 1) {
@@ -424,7 +411,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       sl = sl == SL_FOLD ? SL_RESID : step < cheb ? SL_CHEB : SL_APPLY;
       continue;
     }
-    const bool sums3 = (sl == SL_RESID && last_part) || sl == SL_APPLY || (sl == SL_FRESH && cheb == 1);
+    const bool sums3 = sl == SL_RESID || sl == SL_APPLY || (sl == SL_FRESH && cheb == 1);
     double t3[3] = {0.0, 0.0, 0.0};
     if (sums3) range_sum<3>(prow, NB, E.block0, nbc, t3, dsum);
     else if (sl == SL_FORM) {
@@ -433,10 +420,7 @@ __global__ void __launch_bounds__(kPcgThreads, 2) k_mixed_batch(const MixedBatch
       t3[0] = t1[0];
     }
     if (threadIdx.x == 0) {
-      if (sl == SL_RESID && !last_part) {
-        sc_part = part + 1;
-      } else if (sl == SL_RESID) {
-        sc_part = 0;
+      if (sl == SL_RESID) {
         if (sc_init) sc_bb = t3[2];
         sc_rr = t3[1];
         sc_rr_ref = t3[1];
