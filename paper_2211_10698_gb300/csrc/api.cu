@@ -431,7 +431,8 @@ void case_mixed1_solve(ccm_case c, const MixedSolve& a, const TilePlan& tp, Mixe
   f->resident = tp.resident;
 }
 
-// The resident form (pcg_band.cu); pz and pp0 are FP64 work arrays that mixed solves do not use.
+// The resident form (pcg_band.cu); pz and pp0 are FP64 work arrays that mixed solves do not use.  It lays
+// words, p and e out one element to the left of the other kernels, which clear fp0 and fx when they start.
 void case_band_solve(ccm_case c, const MixedSolve& a, BandSolve* f) {
   *f = BandSolve{};
   f->m = a;

@@ -124,7 +124,7 @@ struct BandTile {
   }
 };
 
-// frame words and e: the quad of cells i .. i + 3 (i a multiple of 4) of row j starts at word i of a
+// frame words, p and e: the quad of cells i .. i + 3 (i a multiple of 4) of row j starts at word i of a
 // row of pitch >= nx + 3 words, 32-byte aligned; a last quad that reaches beyond nx stays in its row
 __device__ __forceinline__ int word(const Geom& g, int i, int j) { return (j + 1) * g.pitch + i; }
 

@@ -2,8 +2,11 @@
 // scaled system K~ = D^-1/2 K D^-1/2) on aligned quads of the padded arrays: padded indices
 // k0 .. k0+3 with k0 a multiple of 4 (the pitch is a multiple of 32, so every row starts a
 // quad).  A row's quads span its interior cells plus the ghost and padding slots beside them;
-// those slots hold zero in every FP32 vector and stay zero (their inputs are zero and their
-// row kind is the identity), so quads are processed whole.  Used by the single-case solve
+// those slots hold zero in every FP32 vector for the whole of a solve (their inputs are zero and
+// their row kind is the identity), so quads are processed whole.  p, s and e are cleared, those
+// slots included, when a solve starts: the band tiles (pcg_band.cu) keep p and e in the same arrays
+// one element to the left and leave cell values in the west ghost column.  The other vectors no
+// kernel writes there.  Used by the single-case solve
 // (pcg_mixed.cu) and the batched one (pcg_batch.cu).
 #pragma once
 #include "pcg_cheb.cuh"
