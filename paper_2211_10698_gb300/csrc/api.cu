@@ -187,8 +187,7 @@ void carve(ccm_case c, Carver& cv) {
   c->fout = cv.take<double>(4);
   c->bar_count = cv.take<unsigned int>(kBarWords);
   c->fxacc = cv.take<unsigned long long>(kFxAccWords);
-  // (mixed solves and periodic sides have no FP64 tiles)
-  c->mail_slots = c->cfg.precision == CCM_MIXED || c->g.px || c->g.py ? 0 : fused_mail_slots_max(c->g.nx, c->g.ny);
+  c->mail_slots = fused_mail_slots_max(c->g.nx, c->g.ny);
   c->mail = cv.take<ulonglong2>(c->mail_slots);
   c->bpart = cv.take<ulonglong2>(2 * kBandTilesMax);
   c->bar_err = cv.take<int>(4);
@@ -1033,9 +1032,6 @@ ccm_status ccm_case_bytes(const ccm_config* cfg, size_t* bytes) {
   tmp.g.nx = cfg->nx;
   tmp.g.ny = cfg->ny;
   tmp.g.pitch = ((cfg->nx + 3) + 31) / 32 * 32;
-  tmp.cfg = *cfg;
-  tmp.g.px = cfg->bc_type[CCM_SIDE_W] == CCM_BC_PERIODIC;
-  tmp.g.py = cfg->bc_type[CCM_SIDE_S] == CCM_BC_PERIODIC;
   Carver dry{nullptr};
   carve(&tmp, dry);
   *bytes = dry.off + 256;
