@@ -178,7 +178,9 @@ enum {
   CCM_F_DY = 13,              /* D_y, one value per v-cell */
   CCM_F_CAP = 16              /* + 9*g + k: capacity k of grid g (read only), g: 0 p, 1 u,
                                  2 v; k: 0 V, 1 X, 2 Y, 3 Ax, 4 Ay, 5 Wx, 6 Wy, 7 Bx, 8 By
-                                 (Ax/Wx at the cell's left face, Ay/Wy at its bottom face) */
+                                 (Ax/Wx at the cell's left face, Ay/Wy at its bottom face).  FP64 cases on
+                                 uniform grids: a V, Ax or Ay that differs from the grid's hx hy, hy or hx by
+                                 the rounding of the abscissas alone is the grid's */
 };
 
 /* Operators for ccm_apply_op.  Inputs/outputs are padded float64 arrays. */
@@ -353,7 +355,7 @@ ccm_status ccm_kernel_timing(ccm_case c, double* poisson_ms, long long* poisson_
 /* Solve the pressure Poisson system of Eq. pm_poisson, K Phi = rhs (rhs on active cells,
  * padded layout, host), starting from the case's PHI field, and store the solution in PHI.
  * With the MIXED precision setting the inner solves run in FP32 and the FP64 residual is
- * refined to tol_p. */
+ * refined to tol_p.  A zero right-hand side has the solution zero, whatever PHI was. */
 ccm_status ccm_solve_pressure(ccm_case c, const double* rhs_host, ccm_solve_stats* stats);
 
 /* Maximum padded size, (ny+3) * pitch elements, that ccm_solve_pressure_noalloc accepts. */

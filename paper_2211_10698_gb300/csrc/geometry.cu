@@ -11,7 +11,9 @@
 //   Wx, Wy         fluid area between the centroid of the left / lower neighbour and the
 //                  cell's own centroid                     (Eqs. volumesecondkindx/y)
 // follow in closed form.  One thread handles one cell of one grid and rebuilds the two
-// neighbours it needs for W, so the kernel has no inter-thread dependence.
+// neighbours it needs for W, so the kernel has no inter-thread dependence.  V, Ax and Ay of uncut
+// cells of a uniform grid are off its spacing by the rounding of the abscissas; with a Snap they are
+// set to it (set_geometry says when and why).
 #include <math.h>
 
 #include "ccm_host.h"

@@ -39,7 +39,7 @@
 // What bounds it: the chain of one iteration, k + 1 block barriers, one L2 hop between SMs (907
 // cycles measured) and the scalars; on large tiles the instructions of the k + 1 passes.  Measured per
 // iteration against the best plan of pcg_mixed.cu and pcg_mixed1.cu: 1024x512, k = 3: 10.8 -> 7.4 us;
-// 2048x1024, k = 2: 27.5 -> 16.4 us; 701x333, Jacobi: 4.9 -> 4.1 us.
+// 2048x1024, k = 3: about 28 -> 16.4 us; 701x333, Jacobi: 4.9 -> 4.1 us.
 #include <algorithm>
 
 #include "batch_common.cuh"
@@ -570,7 +570,7 @@ __device__ __forceinline__ int band_segment(const BandSolve& f, const int tile, 
           }
       }
     };
-    // (many rows: the band's words first, before p takes registers: 2048x1024, k = 2, 17.7 -> 16.4 us
+    // (many rows: the band's words first, before p takes registers: 2048x1024, k = 3, 17.7 -> 16.4 us
     // per iteration; two or more rows' words in flight spill again, 17.3 us and more)
     if (!PG) correct();
 #pragma unroll

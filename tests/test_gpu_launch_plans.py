@@ -13,7 +13,7 @@ def _case(nx, ny, precision, degree=3, autotune=0, bc=None):
     c = I.make_case("plan", nx, ny, (-2.0, 6.0, -2.0, 2.0), I.Geometry(kind=I.GEOM_CIRCLE, cx=0.1, cy=-0.05, r=0.5), re=100.0,
                     cfl=0.5, lref=1.0, bc=bc)
     c.precision, c.autotune, c.tol_p = precision, autotune, 1e-10
-    c.precond, c.cheb_degree = ("chebyshev", degree) if precision == "mixed" else ("jacobi", 1)
+    c.precond, c.cheb_degree = ("chebyshev", degree) if precision == "mixed" and degree > 1 else ("jacobi", 1)
     return c
 
 
@@ -45,6 +45,22 @@ def test_block_counts_and_the_band(nx, ny):
         assert g.launch_plan() == (0, 0, 0, 0, blocks, 0, 0)
         assert not np.array_equal(_phi(g, rhs), built_in)  # other sums: the kernel with a barrier per step
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny,degree,fits", [(2048, 1024, 1, True), (2048, 1024, 3, True), (2048, 1024, 4, False),
+                                               (1792, 952, 8, True), (2048, 1024, 8, False), (2304, 1152, 1, False)])
+def test_where_the_band_ends(nx, ny, degree, fits):
+    """Region rows are at most 15 warps of 9: tile rows and twice the degree."""
+    g = ccm.Case(_case(nx, ny, "mixed", degree))
+    taken = 0
+    for n in range(1, 305):
+        try:
+            g.set_launch_plan((0, 0, 0, 0, ccm.CCM_PLAN_BAND + n, 0, 0))
+            taken += 1
+        except ccm.CcmError:
+            pass
+    g.close()
+    assert taken == (1 if fits else 0)
 
 
 def test_the_band_is_no_fp64_or_closed_box_plan():
